@@ -94,6 +94,79 @@ __device__ __forceinline__ float bilerp_padded(const float* img, int P, int n, f
     return fmaf(aw, bot - top, top);
 }
 
+// ---- packed sampling --------------------------------------------------
+// The fused kernels issue an instruction on more than half of all cycles
+// (about 130 per sample of a grid and iteration), a third of them here, so
+// their sampling uses sm_103's two-wide float instructions: one instruction
+// computes both coordinates of a sample or both rows of a bilinear read, and
+// floor() and its integer come from one rounded addition instead of four
+// trips through the conversion unit.  Every lane performs the operations of
+// the scalar functions above in the same order, so the results are the same
+// bits.  256 candidates x 50 iterations, 128 x 128, 120 views: 35.3 -> 33.5
+// ms (the scalar form of the same floor gains nothing).
+//
+// floor() without the conversion unit: adding 1.5 * 2^23 with rounding
+// towards -inf leaves 1.5 * 2^23 + floor(x) (|x| < 2^22), whose bit pattern
+// is kFloorBits + floor(x).
+constexpr float kFloorBias = 12582912.0f;
+constexpr unsigned kFloorBits = 0x4B400000u;
+
+__device__ __forceinline__ float2 pair(float x) { return make_float2(x, x); }
+// a - b, both lanes
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, pair(-1.0f), a); }
+// a - b c, both lanes, rounded once
+__device__ __forceinline__ float2 sub2_mul(float2 a, float2 b, float2 c) {
+    return __ffma2_rn(b, make_float2(-c.x, -c.y), a);
+}
+
+// A sample's cell in an image of side N padded to pitch P: `frac` the
+// fractions (au, aw), `cell` the padded index of its top left neighbour,
+// `in` whether the footprint touches the image.
+template <int N, int P>
+struct Cell {
+    float2 frac;
+    int cell;
+    bool in;
+    __device__ __forceinline__ explicit Cell(float2 pos) {
+        const float2 t = __fadd2_rd(pos, pair(kFloorBias));
+        frac = sub2(pos, __fadd2_rn(t, pair(-kFloorBias)));
+        const unsigned bj = __float_as_uint(t.x), bi = __float_as_uint(t.y);
+        // floor in [-1, N - 1]: the sample lies in [-1, N)^2 (at -1 every
+        // weight of a pixel inside is 0)
+        in = bj - (kFloorBits - 1) <= (unsigned)N && bi - (kFloorBits - 1) <= (unsigned)N;
+        cell = (int)(bi * P + bj - (kFloorBits - 1u) * (P + 1u));
+    }
+};
+
+// The samples of one ray column, k = k0, k0 + 1, ...: next() returns the
+// position (u, w) that sample_uw gives and moves to the next sample.
+struct ColumnWalk {
+    float2 base, kc;
+    float2 dir;
+    __device__ __forceinline__ ColumnWalk(int k0, int b, float cs, float sn, float c) {
+        const float bc = (float)b - c;
+        base = make_float2(fmaf(bc, cs, c), fmaf(bc, sn, c));
+        kc = pair((float)k0 - c);
+        dir = make_float2(-sn, cs);
+    }
+    __device__ __forceinline__ float2 next() {
+        const float2 pos = __ffma2_rn(kc, dir, base);
+        kc = __fadd2_rn(kc, pair(1.0f));
+        return pos;
+    }
+};
+
+// bilerp_padded at a position.
+template <int N, int P>
+__device__ __forceinline__ float bilerp_pos(const float* img, float2 pos) {
+    const Cell<N, P> x(pos);
+    if (!x.in || !index_ok(x.cell, (long long)P * (N + 1))) return 0.0f;
+    const float* p = img + x.cell;
+    const float2 v0 = make_float2(p[0], p[P]), v1 = make_float2(p[1], p[P + 1]);
+    const float2 tb = __ffma2_rn(pair(x.frac.x), sub2(v1, v0), v0);  // (top, bottom)
+    return fmaf(x.frac.y, tb.y - tb.x, tb.x);
+}
+
 // Transpose of bilerp_padded: add g times each bilinear weight to the four
 // neighbours (non-atomic read-modify-write; callers guarantee that no two
 // threads touch the same pixel concurrently).

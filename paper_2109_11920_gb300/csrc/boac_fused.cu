@@ -238,11 +238,10 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
             float* Uc = QUAD ? Xc + 2 * NN : Xc + NN;
             float* Ur = Uc + N;
             float ps = 0.0f;
+            ColumnWalk walk(k0, lb, cs, sn, c);
 #pragma unroll 8
             for (int s = 0; s < SEG; ++s) {
-                float u, w;
-                sample_uw(k0 + s, lb, cs, sn, c, &u, &w);
-                const float m = bilerp_padded(img0, P, N, u, w);
+                const float m = bilerp_pos<N, P>(img0, walk.next());
                 W[(k0 + s) * WP + lb] = m;
                 ps += m;
             }
@@ -410,6 +409,7 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                 {
                     const float uc = Uc[lb];
                     float acc1 = 0.0f, acc2 = 0.0f;
+                    ColumnWalk walk(k0, lb, cs, sn, c);
 #pragma unroll 2
                     for (int s4 = 0; s4 < SEG; s4 += 4) {
                         const float4 y4 = *reinterpret_cast<const float4*>(Xc + tab_ix(N, k0 + s4, lb));
@@ -417,9 +417,7 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             const int k = k0 + s4 + j;
-                            float u, w;
-                            sample_uw(k, lb, cs, sn, c, &u, &w);
-                            const float f = bilerp_padded(img0, P, N, u, w);
+                            const float f = bilerp_pos<N, P>(img0, walk.next());
                             if (QUAD) W[k * WP + lb] = f;
                             acc1 = fmaf(ex2(yy[j]), f, acc1);
                             acc2 = fmaf(ex2(uc - yy[j]), f, acc2);

@@ -245,14 +245,15 @@ struct SchedSlots {
 };
 
 // The class scatter of scatter_classes (boac_device.cuh), in schedule order.
-// `first` holds this thread's slots of class 0 (loaded by the caller ahead
-// of time); each class's loop loads the next class's slots before it works,
-// so the loads are in flight across the class's work and its barrier.
+// `cur` holds this thread's slots of class 0 (loaded by the caller ahead of
+// time); each class's loop loads the next class's slots before it works, so
+// the loads are in flight across the class's work and its barrier.
 template <int N, int NT, int P, int WP>
 __device__ __forceinline__ void scatter_scheduled(const float* __restrict__ W, float* img1, float cs, float sn,
                                                   float c, const unsigned short* __restrict__ sched,
                                                   SchedSlots<N, NT> cur) {
     constexpr int CE = SchedShape<N>::CLS_ENTRIES;
+    constexpr unsigned kTwo23 = 0x4B000000u;  // bits of 2^23
     static_assert(CE % 64 == 0, "rounds are stored in lane-interleaved pairs");
 #pragma unroll 1
     for (int cls = 0; cls < 9; ++cls) {
@@ -262,25 +263,27 @@ __device__ __forceinline__ void scatter_scheduled(const float* __restrict__ W, f
         for (int h = 0; h < 2 * SchedSlots<N, NT>::KE; ++h) {
             const unsigned v = (cur.e[h >> 1] >> (16 * (h & 1))) & 0xFFFFu;
             if (v == kSchedEmpty) continue;
-            const int k = (int)(v >> 8), b = (int)(v & 255u);
-            if (!index_ok(k, N) || !index_ok(b, N)) continue;
-            float u, w;
-            sample_uw(k, b, cs, sn, c, &u, &w);
+            // k and b as floats without the conversion unit: the byte as the
+            // low mantissa bits of 2^23, less 2^23
+            const unsigned ki = __byte_perm(v, kTwo23, 0x7661), bi = __byte_perm(v, kTwo23, 0x7660);
+            if (!index_ok((int)(ki - kTwo23), N) || !index_ok((int)(bi - kTwo23), N)) continue;
+            const float2 kb = __fadd2_rn(__fadd2_rn(make_float2(__uint_as_float(ki), __uint_as_float(bi)),
+                                                    pair(-8388608.0f)), pair(-c));
             // in (-1, n)^2 by construction: no bounds test (checked builds
             // check the index)
-            const float fj = floorf(u), fi = floorf(w);
-            const float au = u - fj, aw = w - fi;
-            const int idx = ((int)fi + 1) * P + ((int)fj + 1);
-            if (!index_ok(idx, (long long)P * (N + 1))) continue;
-            float* p = img1 + idx;
-            const float g = W[k * WP + b];
-            const float g1 = g * aw, g0 = g - g1;
-            const float g01 = g0 * au, g00 = g0 - g01;
-            const float g11 = g1 * au, g10 = g1 - g11;
-            p[0] += g00;
-            p[1] += g01;
-            p[P] += g10;
-            p[P + 1] += g11;
+            const Cell<N, P> x(make_float2(fmaf(-kb.x, sn, fmaf(kb.y, cs, c)), fmaf(kb.x, cs, fmaf(kb.y, sn, c))));
+            if (!index_ok(x.cell, (long long)P * (N + 1))) continue;
+            float* p = img1 + x.cell;
+            const float g = W[(int)(ki * WP + bi - kTwo23 * (WP + 1u))];
+            const float g1 = __fmul_rn(g, x.frac.y);
+            const float2 row = make_float2(__fsub_rn(g, g1), g1);  // weights of the footprint's rows
+            const float2 au = pair(x.frac.x);
+            const float2 left = __fadd2_rn(make_float2(p[0], p[P]), sub2_mul(row, row, au));
+            const float2 right = __ffma2_rn(row, au, make_float2(p[1], p[P + 1]));
+            p[0] = left.x;
+            p[1] = right.x;
+            p[P] = left.y;
+            p[P + 1] = right.y;
         }
         __syncthreads();
         cur = nxt;
