@@ -639,6 +639,7 @@ struct FusedVariant {
     int (*launch)(const FusedArgs& a, int holders, cudaStream_t st);
     int g;   // CTAs per candidate in the fused kernel's cluster mode (1 otherwise)
     int (*max_clusters)();  // cluster mode: clusters resident at once
+    size_t image_floats;    // one-CTA kernel: F, accumulator and sample buffer of a CTA
 };
 
 // Cluster-mode launches: dynamic shared memory and (16 CTAs) the
@@ -751,13 +752,14 @@ static size_t smem_of(int V) { return fused_smem_bytes<N, NT>(V); }
 template <int N, int NT, bool QUAD>
 static FusedVariant make_variant() {
     return FusedVariant{N, NT, QUAD, 1, smem_of<N, NT>, (const void*)mlem_fused_kernel<N, NT, QUAD>,
-                        fused_launch_t<N, NT, QUAD>, 1, nullptr};
+                        fused_launch_t<N, NT, QUAD>, 1, nullptr, fused_image_floats<N, NT>()};
 }
 
 template <int N, int G>
 static FusedVariant make_split_variant() {
     return FusedVariant{N, 8 * N, true, 1, smem_of<N, 8 * N>, (const void*)mlem_fused_kernel<N, 8 * N, true, G>,
-                        split_launch_t<N, 8 * N, G>, G, split_max_clusters_t<N, 8 * N, G>};
+                        split_launch_t<N, 8 * N, G>, G, split_max_clusters_t<N, 8 * N, G>,
+                        fused_image_floats<N, 8 * N>()};
 }
 
 template <int N, int NB>
@@ -768,7 +770,7 @@ static int band_launch_of(const FusedArgs& a, int clusters, cudaStream_t st) {
 }
 template <int N, int NB>
 static FusedVariant make_band_variant() {
-    return FusedVariant{N, 4 * N, true, NB, band_smem_of<N, NB>, nullptr, band_launch_of<N, NB>, 1, nullptr};
+    return FusedVariant{N, 4 * N, true, NB, band_smem_of<N, NB>, nullptr, band_launch_of<N, NB>, 1, nullptr, 0};
 }
 
 #define BOAC_SHAPES(NV)                                                                        \
@@ -969,12 +971,8 @@ static FusedLayout fused_layout(const boac_geom* g, const FusedVariant* v, int h
     } else {
         l.sens = l.tab + align256(sizeof(float) * ctas * fused_tab_floats(g->n, g->n_views, v->quad, v->g));
         l.img = l.sens + align256(sizeof(float) * ctas * g->n * g->n);
-        // padded F and accumulator, (n+1)(n+2)+1 floats each, and the
-        // n x (n+1) sample buffer, for sides held in global memory
-        const size_t img_floats = fused_global_images(g->n)
-                                      ? 2 * ((size_t)(g->n + 1) * (g->n + 2) + 1) + (size_t)g->n * (g->n + 1)
-                                      : 0;
-        l.geo = l.img + align256(sizeof(float) * ctas * img_floats);
+        // the images and sample buffer of sides held in global memory
+        l.geo = l.img + align256(fused_global_images(g->n) ? sizeof(float) * ctas * v->image_floats : 0);
         l.ready = l.geo;
     }
     l.sched = l.total = l.ready + align256(sizeof(int) * (size_t)B);
