@@ -55,7 +55,7 @@ struct FusedShape {
     // multiple of 32 spreads rotated rows of samples over the banks.
     static constexpr int P = N + 1;
     static constexpr int IMG = (N + 1) * (N + 2) + 1;
-    static constexpr int IMGA = (IMG + 3) & ~3;  // an image's floats, rounded to 16 bytes
+    static constexpr int IMGA = (IMG + kScatterPad + 3) & ~3;  // an image's floats, rounded to 16 bytes
     static constexpr int NN = N * N;
     // Sample-buffer pitch: rows start 16 bytes apart in whole groups, and a
     // quarter-warp's 16-byte row accesses (threads on consecutive rows) fall

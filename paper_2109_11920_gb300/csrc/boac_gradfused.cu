@@ -65,7 +65,7 @@ template <int N>
 struct GradShape {
     static constexpr int NT = 8 * N;
     static constexpr int P = N + 1, WP = N + 1, NN = N * N;
-    static constexpr int IMG = (N + 1) * (N + 2) + 1;
+    static constexpr int IMG = (N + 1) * (N + 2) + 1 + kScatterPad;
     static constexpr int NSEG = 8, SEG = N / 8;
     static constexpr size_t GSTRIDE = 2 * (size_t)NN + 2 * (size_t)N;  // one grid's exponent planes
 };
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(8 * N, 1) grad_fused_kernel(GradFusedArgs a) {
             }
         }
         __syncthreads();
-        scatter_scheduled<N, NT, P, WP>(W, img1, cs, sn, c, gs, sched0);
+        scatter_scheduled<N, NT, P, WP, true>(W, img1, cs, sn, c, gs, sched0);
     };
 
     for (int cand = holder; cand < a.B; cand += n_holders) {
@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(8 * N, 1) grad_fused_kernel(GradFusedArgs a) {
 #pragma unroll 4
             for (int s = 0; s < SEG; ++s) W[(k0 + s) * WP + lb] = __ldcg(Mg + (k0 + s) * N + lb);
             __syncthreads();
-            scatter_scheduled<N, NT, P, WP>(W, img1, csn[2 * gi], csn[2 * gi + 1], c, gs, sched0);
+            scatter_scheduled<N, NT, P, WP, true>(W, img1, csn[2 * gi], csn[2 * gi + 1], c, gs, sched0);
         }
         cluster_sync();
         for (int i = R0 * N + tid; i < R1 * N; i += NT) a.mubar[(size_t)cand * NN + i] = acc_sum(pad(i));

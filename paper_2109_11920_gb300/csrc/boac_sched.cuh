@@ -227,6 +227,10 @@ inline int sched_launch(int n, int V, int ngrid, int wp, unsigned short* sched, 
 const unsigned short* sched_prepare(int n, int V, int ngrid, int wp, unsigned short* ws, cudaStream_t st,
                                     int* status);
 
+// Floats below a padded image (its last padding row starts at (N + 1) P)
+// that the scatter's empty slots may add 0 to: two rows of up to 33 cells.
+constexpr int kScatterPad = 33;
+
 // A thread's words of one class of a grid's schedule (word t = tid + i NT:
 // warp w's lanes hold rounds 2 (w + i NT / 32) and that + 1).
 template <int N, int NT>
@@ -247,34 +251,44 @@ struct SchedSlots {
 // The class scatter of scatter_classes (boac_device.cuh), in schedule order.
 // `cur` holds this thread's slots of class 0 (loaded by the caller ahead of
 // time); each class's loop loads the next class's slots before it works, so
-// the loads are in flight across the class's work and its barrier.
-template <int N, int NT, int P, int WP>
+// the loads are in flight across the class's work and its barrier.  BRANCH:
+// empty slots are skipped; else they add 0 in the padding, which the MLEM
+// kernel prefers (256 candidates x 50 iterations: 31.1 against 31.6 ms) and
+// the gradient kernel, shorter of registers, does not (64 candidates x 10
+// iterations: 8.7 against 8.3 ms).  Preparing a slot, or the next
+// class's first slot, between another slot's loads and stores is slower
+// (31.6 to 36.1 ms).
+template <int N, int NT, int P, int WP, bool BRANCH = false>
 __device__ __forceinline__ void scatter_scheduled(const float* __restrict__ W, float* img1, float cs, float sn,
                                                   float c, const unsigned short* __restrict__ sched,
                                                   SchedSlots<N, NT> cur) {
     constexpr int CE = SchedShape<N>::CLS_ENTRIES;
-    constexpr unsigned kTwo23 = 0x4B000000u;  // bits of 2^23
     static_assert(CE % 64 == 0, "rounds are stored in lane-interleaved pairs");
+    constexpr int kPad = (N + 1) * P;  // the padding row below the image
+    const int pad_cell = kPad + (((int)(threadIdx.x & 31u) - kPad) & 31);  // bank: the lane
 #pragma unroll 1
     for (int cls = 0; cls < 9; ++cls) {
         SchedSlots<N, NT> nxt;
         if (cls < 8) nxt.load(sched + (cls + 1) * CE);
 #pragma unroll
-        for (int h = 0; h < 2 * SchedSlots<N, NT>::KE; ++h) {
-            const unsigned v = (cur.e[h >> 1] >> (16 * (h & 1))) & 0xFFFFu;
-            if (v == kSchedEmpty) continue;
-            // k and b as floats without the conversion unit: the byte as the
-            // low mantissa bits of 2^23, less 2^23
-            const unsigned ki = __byte_perm(v, kTwo23, 0x7661), bi = __byte_perm(v, kTwo23, 0x7660);
-            if (!index_ok((int)(ki - kTwo23), N) || !index_ok((int)(bi - kTwo23), N)) continue;
-            const float2 kb = __fadd2_rn(__fadd2_rn(make_float2(__uint_as_float(ki), __uint_as_float(bi)),
-                                                    pair(-8388608.0f)), pair(-c));
-            // in (-1, n)^2 by construction: no bounds test (checked builds
-            // check the index)
+        for (int i = 0; i < 2 * SchedSlots<N, NT>::KE; ++i) {
+            const unsigned e = cur.e[i >> 1];
+            const bool high = i & 1;
+            bool ok = high ? e < 0xFFFF0000u : (e & 0xFFFFu) != 0xFFFFu;
+            // k and b as floats without the conversion unit: the byte above
+            // the low byte of 2^15's mantissa, less 2^15 (exact: c is a
+            // multiple of 1/2)
+            const unsigned kf = __byte_perm(e, 0x47000000u, high ? 0x7434 : 0x7414);
+            const unsigned bf = __byte_perm(e, 0x47000000u, high ? 0x7424 : 0x7404);
+            const float2 kb = __fadd2_rn(make_float2(__uint_as_float(kf), __uint_as_float(bf)), pair(-32768.0f - c));
             const Cell<N, P> x(make_float2(fmaf(-kb.x, sn, fmaf(kb.y, cs, c)), fmaf(kb.x, cs, fmaf(kb.y, sn, c))));
-            if (!index_ok(x.cell, (long long)P * (N + 1))) continue;
-            float* p = img1 + x.cell;
-            const float g = W[(int)(ki * WP + bi - kTwo23 * (WP + 1u))];
+            const int wi = (int)__dp4a(e, high ? (unsigned)WP << 24 | 1u << 16 : (unsigned)WP << 8 | 1u, 0u);
+            // an entry is in (-1, n)^2 by construction (checked builds check)
+            if (BRANCH && !ok) continue;
+            ok = ok && index_ok(wi, (long long)N * WP) && index_ok(x.cell, (long long)P * (N + 1));
+            float g = 0.0f;
+            if (ok) g = W[wi];
+            float* p = img1 + (ok ? x.cell : pad_cell);
             const float g1 = __fmul_rn(g, x.frac.y);
             const float2 row = make_float2(__fsub_rn(g, g1), g1);  // weights of the footprint's rows
             const float2 au = pair(x.frac.x);
