@@ -104,7 +104,7 @@ template <int N, int NT>
 __host__ __device__ constexpr size_t fused_smem_bytes(int V) {
     using L = FusedShape<N, NT>;
     return sizeof(float) * ((fused_global_images(N) ? 0 : fused_image_floats<N, NT>()) +
-                            4 * L::NSEG * N + 8 * N + 2 * ((V + 1) / 2) * 2) +
+                            4 * L::NSEG * N + 10 * N + 2 * ((V + 1) / 2) * 2) +
            sizeof(double) * 33;
 }
 
@@ -115,6 +115,45 @@ template <int N, int NT>
 constexpr int fused_min_blocks() {
     return (N <= 64 ? 3 : 1) < 1024 / NT ? (N <= 64 ? 3 : 1) : (1024 / NT > 0 ? 1024 / NT : 1);
 }
+
+// A thread's exponents of one grid, from the workspace planes into tensor
+// memory: chunk i is four samples of its column run, or (i >= SEG / 4) of its
+// row run.  A run's exponents lie in the upper half of the columns that its
+// factors will fill: the forward pass reads chunk c (columns SEG + 4 c ..)
+// before it writes that chunk's factors (8 c ..), and those never reach a
+// later chunk's exponents.  As the class scatter's side work the next grid's
+// chunks are loaded one class and stored the next, so their L2 latency, which
+// the forward passes waited for, passes during the scatter.  32 candidates x
+// 20 iterations, 128 x 128, 120 views: 2.13 -> 2.05 ms; 256 x 50: 28.6 -> 28.2.
+template <int N, int SEG, bool QUAD>
+struct ExponentFetch {
+    static constexpr int kRun = SEG / 4, kChunks = (QUAD ? 2 : 1) * kRun;
+    static constexpr int kPerClass = (kChunks + 7) / 8;
+    const float* planes;  // this thread's first sample of its column run
+    unsigned stash;
+    float4 v[kPerClass];
+    __device__ __forceinline__ ExponentFetch(const float* Xc, int k0, int lb, unsigned stash_)
+        : planes(Xc + tab_ix(N, k0, lb)), stash(stash_) {}
+    __device__ __forceinline__ static constexpr int column(int i) {
+        return i < kRun ? SEG + 4 * i : 2 * SEG + SEG + 4 * (i - kRun);
+    }
+    __device__ __forceinline__ float4 load(int i) const {
+        return *reinterpret_cast<const float4*>(planes + 4 * N * i + (i < kRun ? 0 : N * N - 4 * N * kRun));
+    }
+    __device__ __forceinline__ void begin(int cls) {
+#pragma unroll
+        for (int j = 0; j < kPerClass; ++j) {
+            const int i = cls * kPerClass + j, before = i - kPerClass;
+            if (before >= 0 && before < kChunks) tmem_st4(stash + column(before), v[j]);
+            if (i < kChunks) v[j] = load(i);
+        }
+    }
+    // the whole grid at once
+    __device__ __forceinline__ void all() {
+#pragma unroll 4
+        for (int i = 0; i < kChunks; ++i) tmem_st4(stash + column(i), load(i));
+    }
+};
 
 // The scatter schedule of grid gi (images up to 128 x 128 only).
 template <int N>
@@ -148,7 +187,8 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
     float* redr = redc + 2 * NSEG * N;  // [2][NSEG][N] row partial sums
     float* rr = redr + 2 * NSEG * N;    // [4][N] ratios r = S / q per view
     float* Sg = rr + 4 * N;             // [4][N] the grid's sinogram rows (cp.async)
-    float* csn = Sg + 4 * N;            // [V][2]
+    float* Us = Sg + 4 * N;             // [2][N] the grid's whole-ray exponents Uc, Ur (cp.async)
+    float* csn = Us + 2 * N;            // [V][2]
     double* dred = reinterpret_cast<double*>(csn + 2 * ((a.V + 1) / 2) * 2);
 
     const int tid = threadIdx.x;
@@ -162,9 +202,9 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
     const int lb = tid % N, seg = tid / N;
     const int k0 = seg * SEG;
     const size_t gstride = fused_group_floats(N, QUAD);
-    // scatter in schedule order (images up to 128 x 128, schedule present)
+    // scatter in schedule order: images up to 128 x 128
     constexpr int SN = N <= 128 ? N : 128;
-    const bool use_sched = N <= 128 && a.sched != nullptr;
+    constexpr bool use_sched = N <= 128;
 
     for (int v = tid; v < V; v += NT) view_cos_sin(v, V, &csn[2 * v], &csn[2 * v + 1]);
 
@@ -187,14 +227,16 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
         stash = tmem_mine(tmem_addr, tid, kStash);
     }
     // The two factors of each of four samples, from their exponents.
-    auto factors4 = [](const float* y, float total, float (&e)[8]) {
-        const float4 y4 = *reinterpret_cast<const float4*>(y);
-        const float yy[4] = {y4.x, y4.y, y4.z, y4.w};
+    auto factors4 = [](const float (&y)[4], float total, float (&e)[8]) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            e[2 * j] = ex2(yy[j]);
-            e[2 * j + 1] = ex2(total - yy[j]);
+            e[2 * j] = ex2(y[j]);
+            e[2 * j + 1] = ex2(total - y[j]);
         }
+    };
+    auto plane4 = [](const float* p, float (&y)[4]) {
+        const float4 y4 = *reinterpret_cast<const float4*>(p);
+        y[0] = y4.x, y[1] = y4.y, y[2] = y4.z, y[3] = y4.w;
     };
 
     float* tab = a.tab + (size_t)blockIdx.x * fused_tab_floats(N, V, QUAD, G);
@@ -353,7 +395,7 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                 }
             }
             __syncthreads();
-            if (use_sched) scatter_scheduled<SN, NT, P, WP>(W, img1, cs, sn, c, grid_sched<N>(a, gi), sched0);
+            if constexpr (use_sched) scatter_scheduled<SN, NT, P, WP>(W, img1, cs, sn, c, grid_sched<N>(a, gi), sched0);
             else scatter_classes<N, NT, P, WP>(W, img1, cs, sn, c);
         }
         if (tid == 0) {  // second part of a cut candidate: wait for the first
@@ -405,8 +447,35 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
         for (int i = tid; i < IMG; i += NT) img1[i] = 0.0f;
         __syncthreads();
 
+        // What grid gi needs besides its schedule, ahead of its passes: its
+        // sinogram rows and whole-ray exponents copied to shared memory...
+        auto stage = [&](int gi) {
+            for (int t = tid; t < (QUAD ? 4 * N : 2 * N); t += NT) {
+                const int vi = t / N;  // views gi, gi + V/2 (columns), gi + V/4, gi + 3V/4 (rows)
+                const int v = gi + (vi == 0 ? 0 : vi == 1 ? V / 2 : vi == 2 ? V / 4 : 3 * V / 4);
+                copy_async4(Sg + t, S + (size_t)v * N + (t % N));
+            }
+            const float* U = tab + (gi - g0) * gstride + (QUAD ? 2 * NN : NN);
+            for (int t = tid; t < (QUAD ? 2 * N : N); t += NT) copy_async4(Us + t, U + t);
+            copy_async_commit();
+        };
+        // ...and its exponents in tensor memory (or, where they do not fit,
+        // read by the passes)
+        using Fetch = ExponentFetch<N, SEG, QUAD>;
+        auto fetch = [&](int gi) { return Fetch(tab + (gi - g0) * gstride, k0, lb, stash); };
+        auto prepare_now = [&](int gi) {
+            stage(gi);
+            if constexpr (kStashed) {
+                fetch(gi).all();
+                tmem_wait_st();
+            }
+            copy_async_wait_all();
+            __syncthreads();
+        };
+
         // ---- MLEM iterations, then one more forward pass for the score
         double lacc = 0.0;
+        prepare_now(g0);
         for (int it = it0; it <= it1; ++it) {
             const bool scoring = (it == Kc);
             if (it == it1 && !(last && a.L)) break;
@@ -414,36 +483,31 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                 const float cs = csn[2 * gi], sn = csn[2 * gi + 1];
                 const float* Xc = tab + (gi - g0) * gstride;
                 const float* XrT = Xc + NN;
-                const float* Uc = QUAD ? Xc + 2 * NN : Xc + NN;
-                const float* Ur = Uc + N;
+                const int gn = gi + 1 < g1 ? gi + 1 : g0;
                 {   // the next grid's exponent planes are read from DRAM
                     // once per iteration: start that read now (one 128-byte
                     // line per thread, 2 n^2 floats per grid)
-                    const int gn = gi + 1 < g1 ? gi + 1 : g0;
                     const float* nxt = tab + (gn - g0) * gstride;
                     constexpr int kLines = (int)((2 * (size_t)NN * sizeof(float) + 127) / 128);
                     for (int l = tid; l < (QUAD ? kLines : kLines / 2); l += NT) prefetch_l2(nxt + 32 * l);
                 }
-                const int vc1 = gi, vc2 = gi + V / 2;           // column views
-                const int vr1 = gi + V / 4, vr2 = gi + 3 * V / 4;  // row views (QUAD)
-                // the grid's sinogram rows, copied to shared memory while the
-                // forward passes run (waited for before the ratio step)
-                for (int t = tid; t < (QUAD ? 4 * N : 2 * N); t += NT) {
-                    const int vi = t / N, v = vi == 0 ? vc1 : vi == 1 ? vc2 : vi == 2 ? vr1 : vr2;
-                    copy_async4(Sg + t, S + (size_t)v * N + (t % N));
-                }
-                copy_async_commit();
-                // forward, column views: sample F on the grid.  (The column
-                // and row passes and the column weights unroll by 8: fully
-                // unrolled they spill at 64 registers; measured +7.8 %.)
+                // forward, column views: sample F on the grid.  (Unrolled by
+                // 8 samples; the whole run at once takes 31.7 instead of 28.2
+                // ms, the row pass is best unrolled by 16.)
                 {
-                    const float uc = Uc[lb];
+                    const float uc = Us[lb];
                     float acc1 = 0.0f, acc2 = 0.0f;
                     ColumnWalk walk(k0, lb, cs, sn, c);
 #pragma unroll 2
                     for (int s4 = 0; s4 < SEG; s4 += 4) {
-                        float e[8];
-                        factors4(Xc + tab_ix(N, k0 + s4, lb), uc, e);
+                        float y[4], e[8];
+                        if constexpr (kStashed) {
+                            tmem_ld4(stash + SEG + s4, y);
+                            tmem_wait_ld(y);
+                        } else {
+                            plane4(Xc + tab_ix(N, k0 + s4, lb), y);
+                        }
+                        factors4(y, uc, e);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             const int k = k0 + s4 + j;
@@ -459,14 +523,17 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                 }
                 if (QUAD) {  // forward, row views: the samples back from W
                     __syncthreads();
-                    const float ur = Ur[lb];
+                    const float ur = Us[N + lb];
                     float acc3 = 0.0f, acc4 = 0.0f;
-#pragma unroll 2
+#pragma unroll 4
                     for (int s4 = 0; s4 < SEG; s4 += 4) {
+                        float y[4], e[8];
+                        if constexpr (kStashed) tmem_ld4(stash + 3 * SEG + s4, y);
+                        else plane4(XrT + tab_ix(N, k0 + s4, lb), y);
                         const float4 f4 = *reinterpret_cast<const float4*>(W + lb * WP + k0 + s4);
                         const float ff[4] = {f4.x, f4.y, f4.z, f4.w};
-                        float e[8];
-                        factors4(XrT + tab_ix(N, k0 + s4, lb), ur, e);
+                        if constexpr (kStashed) tmem_wait_ld(y);
+                        factors4(y, ur, e);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             acc3 = fmaf(e[2 * j], ff[j], acc3);
@@ -477,12 +544,11 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                     redr[seg * N + lb] = acc3;
                     redr[(NSEG + seg) * N + lb] = acc4;
                 }
-                copy_async_wait_all();
                 if constexpr (kStashed) tmem_wait_st();
                 __syncthreads();
                 // q, then r = S / q (or the Eq. 5 terms when scoring)
                 for (int t = tid; t < (QUAD ? 4 * N : 2 * N); t += NT) {  // one ray per thread
-                    const int j = t % N, vi = t / N;  // views vc1, vc2, vr1, vr2
+                    const int j = t % N, vi = t / N;
                     const float* rp = (vi >= 2 ? redr : redc) + ((vi & 1) ? NSEG * N : 0);
                     float q = 0.0f;
 #pragma unroll
@@ -493,13 +559,18 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                     else rr[vi * N + j] = q > 0.0f ? Sv / q : 0.0f;
                 }
                 __syncthreads();
-                if (scoring) continue;
+                if (scoring) {
+                    prepare_now(gn);
+                    continue;
+                }
+                stage(gn);
                 SchedSlots<SN, NT> sched0;  // in flight during the weight passes
                 if (use_sched) sched0.load(grid_sched<N>(a, gi));
                 // back-projection weights of the grid's views, from the stashed
                 // factors
                 {
                     const float r1 = dx * rr[lb], r2 = dx * rr[N + lb];
+                    [[maybe_unused]] const float uc = kStashed ? 0.0f : Xc[(QUAD ? 2 * NN : NN) + lb];
 #pragma unroll 2
                     for (int s4 = 0; s4 < SEG; s4 += 4) {
                         float e[8];
@@ -507,7 +578,9 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                             tmem_ld8(stash + 2 * s4, e);
                             tmem_wait_ld(e);
                         } else {
-                            factors4(Xc + tab_ix(N, k0 + s4, lb), Uc[lb], e);
+                            float y[4];
+                            plane4(Xc + tab_ix(N, k0 + s4, lb), y);
+                            factors4(y, uc, e);
                         }
 #pragma unroll
                         for (int j = 0; j < 4; ++j) W[(k0 + s4 + j) * WP + lb] = fmaf(e[2 * j], r1, e[2 * j + 1] * r2);
@@ -516,6 +589,7 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                 if (QUAD) {
                     __syncthreads();
                     const float r3 = dx * rr[2 * N + lb], r4 = dx * rr[3 * N + lb];
+                    [[maybe_unused]] const float ur = kStashed ? 0.0f : Xc[2 * NN + N + lb];
 #pragma unroll 2
                     for (int s4 = 0; s4 < SEG; s4 += 4) {
                         float e[8];
@@ -525,7 +599,9 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                             tmem_ld8(stash + 2 * (SEG + s4), e);
                             tmem_wait_ld(e);
                         } else {
-                            factors4(XrT + tab_ix(N, k0 + s4, lb), Ur[lb], e);
+                            float y[4];
+                            plane4(XrT + tab_ix(N, k0 + s4, lb), y);
+                            factors4(y, ur, e);
                         }
                         v.x += fmaf(e[0], r3, e[1] * r4);
                         v.y += fmaf(e[2], r3, e[3] * r4);
@@ -534,9 +610,13 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                         *w4 = v;
                     }
                 }
+                copy_async_wait_all();
                 __syncthreads();
-                if (use_sched) scatter_scheduled<SN, NT, P, WP>(W, img1, cs, sn, c, grid_sched<N>(a, gi), sched0);
-                else scatter_classes<N, NT, P, WP>(W, img1, cs, sn, c);
+                if constexpr (use_sched)
+                    scatter_scheduled<SN, NT, P, WP, false>(W, img1, cs, sn, c, grid_sched<N>(a, gi), sched0, fetch(gn));
+                else
+                    scatter_classes<N, NT, P, WP>(W, img1, cs, sn, c);
+                if constexpr (kStashed) tmem_wait_st();
             }
             if (scoring) break;
             if constexpr (G > 1) {

@@ -261,10 +261,17 @@ struct SchedSlots {
 // iterations: 8.7 against 8.3 ms).  Preparing a slot, or the next
 // class's first slot, between another slot's loads and stores is slower
 // (31.6 to 36.1 ms).
-template <int N, int NT, int P, int WP, bool BRANCH = false>
+//
+// `side` is work that each thread does beside the classes (NoSideWork:
+// none), begin(cls) at the start of class cls.
+struct NoSideWork {
+    __device__ __forceinline__ void begin(int) {}
+};
+
+template <int N, int NT, int P, int WP, bool BRANCH = false, class Side = NoSideWork>
 __device__ __forceinline__ void scatter_scheduled(const float* __restrict__ W, float* img1, float cs, float sn,
                                                   float c, const unsigned short* __restrict__ sched,
-                                                  SchedSlots<N, NT> cur) {
+                                                  SchedSlots<N, NT> cur, Side side = Side()) {
     constexpr int CE = SchedShape<N>::CLS_ENTRIES;
     static_assert(CE % 64 == 0, "rounds are stored in lane-interleaved pairs");
     constexpr int kPad = (N + 1) * P;  // the padding row below the image
@@ -273,6 +280,7 @@ __device__ __forceinline__ void scatter_scheduled(const float* __restrict__ W, f
     for (int cls = 0; cls < 9; ++cls) {
         SchedSlots<N, NT> nxt;
         if (cls < 8) nxt.load(sched + (cls + 1) * CE);
+        side.begin(cls);
 #pragma unroll
         for (int i = 0; i < 2 * SchedSlots<N, NT>::KE; ++i) {
             const unsigned e = cur.e[i >> 1];

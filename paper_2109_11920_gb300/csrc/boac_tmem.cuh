@@ -57,6 +57,18 @@ __device__ __forceinline__ void tmem_ld8(unsigned addr, float (&v)[8]) {
                  : "r"(addr)
                  : "memory");
 }
+// Four floats, likewise.
+__device__ __forceinline__ void tmem_st4(unsigned addr, float4 v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y),
+                 "f"(v.z), "f"(v.w)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(unsigned addr, float (&v)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                 : "r"(addr)
+                 : "memory");
+}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // The loaded values are used only after the wait: they pass through it.
 __device__ __forceinline__ void tmem_wait_ld(float (&a)[8]) {
@@ -65,10 +77,9 @@ __device__ __forceinline__ void tmem_wait_ld(float (&a)[8]) {
                  :
                  : "memory");
 }
-__device__ __forceinline__ void tmem_wait_ld(float (&a)[8], float (&b)[8]) {
+__device__ __forceinline__ void tmem_wait_ld(float (&a)[4]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]),
-                   "+f"(b[0]), "+f"(b[1]), "+f"(b[2]), "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7])
+                 : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3])
                  :
                  : "memory");
 }
