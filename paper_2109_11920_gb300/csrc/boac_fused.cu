@@ -100,12 +100,20 @@ __host__ __device__ constexpr size_t fused_image_floats() {
     return 2 * (size_t)L::IMGA + (size_t)N * L::WP;
 }
 
+// A 96 x 96 CTA takes all of its SM's tensor memory (288 of the 512 columns
+// used, and allocations are powers of two) but only half of its shared memory.
+// It asks for enough of the latter that no 64 x 64 CTA of another launch (56
+// KB, 128 columns) fits beside it, where one of the two would wait for the
+// other's tensor memory until that kernel ends.
+constexpr size_t kSoleSmem = 176 * 1024;
+
 template <int N, int NT>
 __host__ __device__ constexpr size_t fused_smem_bytes(int V) {
     using L = FusedShape<N, NT>;
-    return sizeof(float) * ((fused_global_images(N) ? 0 : fused_image_floats<N, NT>()) +
-                            4 * L::NSEG * N + 10 * N + 2 * ((V + 1) / 2) * 2) +
-           sizeof(double) * 33;
+    const size_t need = sizeof(float) * ((fused_global_images(N) ? 0 : fused_image_floats<N, NT>()) +
+                                         4 * L::NSEG * N + 10 * N + 2 * ((V + 1) / 2) * 2) +
+                        sizeof(double) * 33;
+    return N == 96 && need < kSoleSmem ? kSoleSmem : need;
 }
 
 // CTAs per SM the register allocation is sized for: as many as shared memory
