@@ -334,7 +334,11 @@ __global__ void __launch_bounds__(4 * N, N == 64 ? 4 : (N == 128 && NB > 2) ? 2 
     using L = BandSmem<N, NB>;
     constexpr int NT = S::NT, H = S::H, P = S::P, BIMG = S::BIMG, WP = S::WP, TC = S::TC;
     constexpr float kLog2e = 1.44269504088896340736f;
-    if (*a.geo_bad) return;  // set before this launch: uniform over all CTAs
+    class_begin(a);
+    if (*a.geo_bad) {  // set before this launch: uniform over all CTAs
+        class_end(a);
+        return;
+    }
 
     cg::cluster_group cl = cg::this_cluster();
     const int r = (int)cl.block_rank();
@@ -783,6 +787,7 @@ __global__ void __launch_bounds__(4 * N, N == 64 ? 4 : (N == 128 && NB > 2) ? 2 
         if (!last && r == 0 && tid == 0 && cand != a.withhold)
             asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(a.ready + cand), "r"(1) : "memory");
     }
+    class_end(a);
 }
 
 // ---------------------------------------------------------------- host side
@@ -877,27 +882,38 @@ int band_max_clusters(int n, int nb) {
 }
 
 template <int N, int NB>
+static int band_prepare_t(const FusedArgs& a, cudaStream_t st) {
+    if (cudaMemsetAsync(a.geo_bad, 0, sizeof(int), st) != cudaSuccess) return launch_status();
+    band_records_kernel<N, NB><<<dim3(a.V / 4, NB), N, 0, st>>>(a.V, const_cast<int*>(a.geo), a.geo_bad);
+    return launch_status();
+}
+
+template <int N, int NB>
 static int band_launch_t(const FusedArgs& a, int clusters, cudaStream_t st) {
     int s = set_smem_attr<N, NB>();
     if (s != BOAC_OK) return s;
-    if (cudaMemsetAsync(a.geo_bad, 0, sizeof(int), st) != cudaSuccess) return launch_status();
-    band_records_kernel<N, NB><<<dim3(a.V / 4, NB), N, 0, st>>>(a.V, const_cast<int*>(a.geo), a.geo_bad);
-    s = launch_status();
-    if (s != BOAC_OK) return s;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = NB;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    overlap_attribute(&attr[1], a);
     cfg.gridDim = dim3((unsigned)(clusters * NB), 1, 1);
     cfg.blockDim = dim3(BandShape<N, NB>::NT, 1, 1);
     cfg.dynamicSmemBytes = BandSmem<N, NB>::BYTES;
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     if (cudaLaunchKernelEx(&cfg, mlem_band_kernel<N, NB>, a) != cudaSuccess) return launch_status();
     return launch_status();
+}
+
+int band_prepare(int n, int nb, const FusedArgs& a, cudaStream_t st) {
+#define X(NV, BV) if (n == NV && nb == BV) return band_prepare_t<NV, BV>(a, st);
+    BOAC_BAND_CASES(X)
+#undef X
+    return BOAC_EUNSUPPORTED;
 }
 
 int band_launch(int n, int nb, const FusedArgs& a, int clusters, cudaStream_t st) {

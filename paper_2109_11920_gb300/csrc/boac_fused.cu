@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
     constexpr int NSEG = Lay::NSEG, SEG = Lay::SEG;
     constexpr float kLog2e = 1.44269504088896340736f;
 
+    class_begin(a);
     extern __shared__ __align__(16) float smem[];
     float* const img_base = fused_global_images(N)
                                 ? a.img + (size_t)blockIdx.x * fused_image_floats<N, NT>()
@@ -701,6 +702,7 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
         __syncthreads();
         if (tid < 32) tmem_free<kTmemCols>(tmem_addr);
     }
+    class_end(a);
 }
 
 // ---------------------------------------------------------------- host side
@@ -723,6 +725,9 @@ struct FusedVariant {
     int nb;  // CTAs per candidate in the band kernel's cluster (1 otherwise)
     size_t (*smem)(int V);
     const void* func;
+    // what the geometry needs before the kernel: the scatter schedule (its
+    // place left in a->sched) or the ray-run records
+    int (*prepare)(FusedArgs* a, cudaStream_t st);
     // `holders`: CTAs (nb == 1, g == 1) or clusters that share the work
     int (*launch)(const FusedArgs& a, int holders, cudaStream_t st);
     int g;   // CTAs per candidate in the fused kernel's cluster mode (1 otherwise)
@@ -767,6 +772,15 @@ static cudaLaunchConfig_t split_config(int clusters, int V, cudaStream_t st, cud
     return cfg;
 }
 
+template <int N, int NT, bool QUAD>
+static int fused_prepare_t(FusedArgs* a, cudaStream_t st) {
+    int s = BOAC_OK;
+    if constexpr (N <= 128)
+        a->sched = sched_prepare(N, a->V, QUAD ? a->V / 4 : a->V / 2, FusedShape<N, NT>::WP,
+                                 const_cast<unsigned short*>(a->sched), st, &s);
+    return s;
+}
+
 template <int N, int NT, int G>
 static int split_max_clusters_t() {
     constexpr int kDev = 64;
@@ -796,15 +810,11 @@ template <int N, int NT, int G>
 static int split_launch_t(const FusedArgs& a, int clusters, cudaStream_t st) {
     int s = split_attrs<N, NT, G>();
     if (s != BOAC_OK) return s;
-    FusedArgs b = a;
-    if (b.sched) {  // the scatter schedule of this geometry, then the kernel
-        b.sched = sched_prepare(N, b.V, b.V / 4, FusedShape<N, NT>::WP, const_cast<unsigned short*>(a.sched), st,
-                                &s);
-        if (s != BOAC_OK) return s;
-    }
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = split_config<N, NT, G>(clusters, b.V, st, attr);
-    if (cudaLaunchKernelEx(&cfg, mlem_fused_kernel<N, NT, true, G>, b) != cudaSuccess) return launch_status();
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = split_config<N, NT, G>(clusters, a.V, st, attr);
+    overlap_attribute(&attr[1], a);
+    cfg.numAttrs = 2;
+    if (cudaLaunchKernelEx(&cfg, mlem_fused_kernel<N, NT, true, G>, a) != cudaSuccess) return launch_status();
     return launch_status();
 }
 
@@ -821,16 +831,16 @@ static int fused_launch_t(const FusedArgs& a, int slots, cudaStream_t st) {
             return launch_status();
         attr_set[dev] = true;
     }
-    FusedArgs b = a;
-    if constexpr (N <= 128) {
-        if (b.sched) {  // the scatter schedule of this geometry, then the kernel
-            int s = BOAC_OK;
-            b.sched = sched_prepare(N, b.V, QUAD ? b.V / 4 : b.V / 2, FusedShape<N, NT>::WP,
-                                    const_cast<unsigned short*>(a.sched), st, &s);
-            if (s != BOAC_OK) return s;
-        }
-    }
-    mlem_fused_kernel<N, NT, QUAD><<<slots, NT, fused_smem_bytes<N, NT>(b.V), st>>>(b);
+    cudaLaunchAttribute attr[1];
+    overlap_attribute(&attr[0], a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)slots, 1, 1);
+    cfg.blockDim = dim3(NT, 1, 1);
+    cfg.dynamicSmemBytes = fused_smem_bytes<N, NT>(a.V);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, mlem_fused_kernel<N, NT, QUAD>, a) != cudaSuccess) return launch_status();
     return launch_status();
 }
 
@@ -840,25 +850,31 @@ static size_t smem_of(int V) { return fused_smem_bytes<N, NT>(V); }
 template <int N, int NT, bool QUAD>
 static FusedVariant make_variant() {
     return FusedVariant{N, NT, QUAD, 1, smem_of<N, NT>, (const void*)mlem_fused_kernel<N, NT, QUAD>,
-                        fused_launch_t<N, NT, QUAD>, 1, nullptr, fused_image_floats<N, NT>()};
+                        fused_prepare_t<N, NT, QUAD>, fused_launch_t<N, NT, QUAD>, 1, nullptr,
+                        fused_image_floats<N, NT>()};
 }
 
 template <int N, int G>
 static FusedVariant make_split_variant() {
     return FusedVariant{N, 8 * N, true, 1, smem_of<N, 8 * N>, (const void*)mlem_fused_kernel<N, 8 * N, true, G>,
-                        split_launch_t<N, 8 * N, G>, G, split_max_clusters_t<N, 8 * N, G>,
+                        fused_prepare_t<N, 8 * N, true>, split_launch_t<N, 8 * N, G>, G, split_max_clusters_t<N, 8 * N, G>,
                         fused_image_floats<N, 8 * N>()};
 }
 
 template <int N, int NB>
 static size_t band_smem_of(int) { return band_smem_bytes(N, NB); }
 template <int N, int NB>
+static int band_prepare_of(FusedArgs* a, cudaStream_t st) {
+    return band_prepare(N, NB, *a, st);
+}
+template <int N, int NB>
 static int band_launch_of(const FusedArgs& a, int clusters, cudaStream_t st) {
     return band_launch(N, NB, a, clusters, st);
 }
 template <int N, int NB>
 static FusedVariant make_band_variant() {
-    return FusedVariant{N, 4 * N, true, NB, band_smem_of<N, NB>, nullptr, band_launch_of<N, NB>, 1, nullptr, 0};
+    return FusedVariant{N, 4 * N, true, NB, band_smem_of<N, NB>, nullptr, band_prepare_of<N, NB>,
+                        band_launch_of<N, NB>, 1, nullptr, 0};
 }
 
 #define BOAC_SHAPES(NV)                                                                        \
@@ -1040,7 +1056,8 @@ static int variant_occupancy(const FusedVariant* v, int V) {
 //   images     one-CTA kernel, n > 128: padded F / accumulator / sample
 //              buffer per CTA; cluster kernel: the record kernel's flag and
 //              the ray-run records of every (band, grid)
-//   ready      one flag per candidate (the work split's hand-over)
+//   ready      one flag per candidate (the work split's hand-over), then the
+//              count of finished CTAs (ragged batches)
 //   sched      one-CTA kernel, n <= 128: the scatter schedule (geometry only)
 struct FusedLayout {
     size_t status, tab, sens, img, geo, ready, sched, total;
@@ -1063,7 +1080,7 @@ static FusedLayout fused_layout(const boac_geom* g, const FusedVariant* v, int h
         l.geo = l.img + align256(fused_global_images(g->n) ? sizeof(float) * ctas * v->image_floats : 0);
         l.ready = l.geo;
     }
-    l.sched = l.total = l.ready + align256(sizeof(int) * (size_t)B);
+    l.sched = l.total = l.ready + align256(sizeof(int) * ((size_t)B + 1));
     if (v->nb == 1 && g->n <= 128) l.total = l.sched + sched_bytes(g->n, v->quad ? g->n_views / 4 : g->n_views / 2);
     return l;
 }
@@ -1125,6 +1142,8 @@ static FusedArgs base_args(const boac_geom* g, const float* mu, const float* S, 
     a.wait_cycles = wait_cycles();
     a.withhold = -1;
     a.sched = l.total > l.sched ? reinterpret_cast<const unsigned short*>(ws + l.sched) : nullptr;
+    a.overlap = 0;
+    a.done = a.ready + B;
     return a;
 }
 
@@ -1150,7 +1169,8 @@ static int launch_uniform(const boac_geom* g, const FusedVariant* v, int slots, 
         a.lgS = lgamma_sum(g->n_views * g->n_bins, S, reinterpret_cast<double*>(ws + l.status + 8), st);
     }
     BOAC_RANGE("fused MLEM: set-up, iterations, score");
-    return v->launch(a, grid, st);
+    const int s = v->prepare(&a, st);
+    return s == BOAC_OK ? v->launch(a, grid, st) : s;
 }
 
 // ---------------------------------------------------------------- ragged
@@ -1159,11 +1179,64 @@ static int launch_uniform(const boac_geom* g, const FusedVariant* v, int slots, 
 // fused layout (without its own status word).
 struct RaggedPlan {
     int cls_count[kMaxRaggedClasses];
+    long long units[kMaxRaggedClasses], longest[kMaxRaggedClasses];
+    double chain[kMaxRaggedClasses];  // modelled time of the class's busiest CTA
+    bool shares_sm[kMaxRaggedClasses];  // several of the class's CTAs fit an SM
     int slots[kMaxRaggedClasses];
     const FusedVariant* var[kMaxRaggedClasses];
     size_t desc_off[kMaxRaggedClasses], start_off[kMaxRaggedClasses], layout_off[kMaxRaggedClasses];
     size_t total;
 };
+
+// Shares the SMs out among the classes, whose kernels run at once.  A class
+// of one-CTA candidates needs at least the SMs that finish its work in the
+// time T of the longest chain: T starts at the larger of the longest
+// candidate's time and the even share of all work, and grows until the
+// classes fit the GPU together.  Time per sample grid, measured: 11.1 us at
+// 128 x 128 and 5.3 us at 64 x 64, that is 0.47 ns per sample and as much as
+// 7200 samples for its barriers; two views per grid 0.85 times that (6.5 us
+// at 96 x 96); two CTAs on an SM take 1.45 times the time of one.  A split
+// only decides which CTA runs which iterations, never what they compute.
+static void ragged_share(const boac_geom* classes, int n_classes, RaggedPlan* pl) {
+    const int sms = sm_count();
+    double cost[kMaxRaggedClasses], T = 0.0, work = 0.0;
+    int per_sm[kMaxRaggedClasses], classes_in_use = 0;
+    for (int c = 0; c < n_classes; ++c) {
+        const FusedVariant* v = pl->var[c];
+        const boac_geom& g = classes[c];
+        per_sm[c] = v->nb > 1 || v->g > 1 ? 0 : variant_occupancy(v, g.n_views);
+        cost[c] = (v->quad ? g.n_views / 4 : 0.85 * (g.n_views / 2)) * ((double)g.n * g.n + 7200.0) *
+                  (per_sm[c] > 1 ? 1.0 + 0.45 * (per_sm[c] - 1) : 1.0);
+        pl->chain[c] = 0.0;
+        pl->shares_sm[c] = per_sm[c] > 1;
+        if (pl->cls_count[c] == 0) continue;
+        ++classes_in_use;
+        const int ctas = v->nb > 1 ? v->nb : v->g;
+        pl->chain[c] = cost[c] / ctas * split_cap(pl->units[c], pl->longest[c], pl->slots[c]);
+        if (per_sm[c] == 0) continue;  // clusters: as many as are resident, where SMs are free
+        if (cost[c] * pl->longest[c] > T) T = cost[c] * pl->longest[c];
+        work += cost[c] * pl->units[c] / per_sm[c];
+    }
+    if (classes_in_use < 2 || sms <= 0 || work <= 0.0) return;
+    if (work / sms > T) T = work / sms;
+    for (int step = 0; step < 200; ++step, T *= 1.01) {
+        int need[kMaxRaggedClasses], used = 0;
+        for (int c = 0; c < n_classes; ++c) {
+            need[c] = 0;
+            if (pl->cls_count[c] == 0 || per_sm[c] == 0) continue;
+            const double n = ceil(pl->units[c] * cost[c] / T);
+            need[c] = n < pl->slots[c] ? (int)n : pl->slots[c];
+            used += (need[c] + per_sm[c] - 1) / per_sm[c];
+        }
+        if (used > sms) continue;
+        for (int c = 0; c < n_classes; ++c)
+            if (need[c] > 0) {
+                pl->slots[c] = need[c];
+                pl->chain[c] = cost[c] * split_cap(pl->units[c], pl->longest[c], need[c]);
+            }
+        return;
+    }
+}
 
 static int ragged_plan(const boac_geom* classes, int n_classes, const boac_ragged_cand* cands, int B,
                        const int* config, RaggedPlan* pl) {
@@ -1171,12 +1244,16 @@ static int ragged_plan(const boac_geom* classes, int n_classes, const boac_ragge
     for (int c = 0; c < n_classes; ++c) {
         if (!geom_ok(&classes[c]) || classes[c].n_views % 2) return BOAC_EINVAL;
         pl->cls_count[c] = 0;
+        pl->units[c] = pl->longest[c] = 0;
     }
     for (int b = 0; b < B; ++b) {
         const boac_ragged_cand& d = cands[b];
         if (d.cls < 0 || d.cls >= n_classes || d.K < 0 || d.mu_off < 0 || d.S_off < 0 || d.F_off < 0)
             return BOAC_EINVAL;
         pl->cls_count[d.cls]++;
+        const long long len = d.K > 0 ? d.K : 1;
+        pl->units[d.cls] += len;
+        if (len > pl->longest[d.cls]) pl->longest[d.cls] = len;
     }
     size_t off = 256;
     for (int c = 0; c < n_classes; ++c) {
@@ -1187,6 +1264,10 @@ static int ragged_plan(const boac_geom* classes, int n_classes, const boac_ragge
         const int cnt = pl->cls_count[c];
         pl->slots[c] = cnt ? variant_holders(&classes[c], pl->var[c], cnt) : 0;
         if (cnt && pl->slots[c] <= 0) return BOAC_ECUDA;
+    }
+    ragged_share(classes, n_classes, pl);
+    for (int c = 0; c < n_classes; ++c) {
+        const int cnt = pl->cls_count[c];
         pl->desc_off[c] = off;
         off += align256(sizeof(RaggedDesc) * (size_t)cnt);
         pl->start_off[c] = off;
@@ -1279,7 +1360,8 @@ extern "C" int boac_test_mlem_handover(const boac_geom* g, const float* mu, cons
     if (cudaMemsetAsync(base + l.status, 0, sizeof(int), st) != cudaSuccess ||
         cudaMemsetAsync(base + l.ready, 0, sizeof(int) * (size_t)B, st) != cudaSuccess)
         return launch_status();
-    return v->launch(a, grid, st);
+    const int ps = v->prepare(&a, st);
+    return ps == BOAC_OK ? v->launch(a, grid, st) : ps;
 }
 
 extern "C" int boac_workspace_status(const void* ws, size_t ws_bytes, int* status) {
@@ -1344,27 +1426,41 @@ extern "C" int boac_mlem_ragged_run(const boac_geom* classes, int n_classes,
     char* base = static_cast<char*>(ws);
     cudaStream_t st = as_stream(stream);
     if (cudaMemsetAsync(base, 0, sizeof(int), st) != cudaSuccess) return launch_status();
-    // units and longest candidate per class (the same order as prepare's)
-    long long units[kMaxRaggedClasses] = {0}, longest[kMaxRaggedClasses] = {0};
-    for (int b = 0; b < B; ++b) {
-        const long long len = cands[b].K > 0 ? cands[b].K : 1;
-        units[cands[b].cls] += len;
-        if (len > longest[cands[b].cls]) longest[cands[b].cls] = len;
-    }
+    // What every class's kernel needs first, then the kernels, each free to
+    // start beside the ones before it: one after the other they take the sum
+    // of the classes' longest chains (256 candidates of three sizes, 20 to 80
+    // iterations: 57.0 ms, together 28.8).  The longest chain goes first, but
+    // CTAs that share an SM last: on an empty GPU each would be given an SM of
+    // its own and keep the larger CTAs off it.
+    FusedArgs args[kMaxRaggedClasses];
+    int grids[kMaxRaggedClasses], order[kMaxRaggedClasses], used = 0;
     for (int c = 0; c < n_classes; ++c) {
         const int cnt = pl.cls_count[c];
         if (cnt == 0) continue;
+        int at = used++;
+        auto before = [&](int x, int y) {
+            return pl.shares_sm[x] != pl.shares_sm[y] ? pl.shares_sm[y] : pl.chain[x] > pl.chain[y];
+        };
+        for (; at > 0 && before(c, order[at - 1]); --at) order[at] = order[at - 1];
+        order[at] = c;
         const FusedLayout l = fused_layout(&classes[c], pl.var[c], pl.slots[c], cnt);
         char* cbase = base + pl.layout_off[c];
         FusedArgs a = base_args(&classes[c], mu_pool, S_pool, 0, F_pool, 0, cnt, L, include_lgamma, cbase, l);
         a.desc = reinterpret_cast<const RaggedDesc*>(base + pl.desc_off[c]);
         a.job_start = reinterpret_cast<const long long*>(base + pl.start_off[c]);
         a.status = reinterpret_cast<int*>(base);  // one status word for the call
-        a.cap = split_cap(units[c], longest[c], pl.slots[c]);
-        const int grid = (int)((units[c] + a.cap - 1) / a.cap);
-        if (cudaMemsetAsync(cbase + l.ready, 0, sizeof(int) * (size_t)cnt, st) != cudaSuccess)
+        a.cap = split_cap(pl.units[c], pl.longest[c], pl.slots[c]);
+        grids[c] = (int)((pl.units[c] + a.cap - 1) / a.cap);
+        if (cudaMemsetAsync(cbase + l.ready, 0, sizeof(int) * ((size_t)cnt + 1), st) != cudaSuccess)
             return launch_status();
-        s = pl.var[c]->launch(a, grid, st);
+        s = pl.var[c]->prepare(&a, st);
+        if (s != BOAC_OK) return s;
+        args[c] = a;
+    }
+    for (int i = 0; i < used; ++i) {
+        const int c = order[i];
+        args[c].overlap = (i + 1 < used ? FusedArgs::kTrigger : 0) | (i > 0 ? FusedArgs::kJoin : 0);
+        s = pl.var[c]->launch(args[c], grids[c], st);
         if (s != BOAC_OK) return s;
     }
     return BOAC_OK;

@@ -67,7 +67,33 @@ struct FusedArgs {
     // flag the record kernel sets if a run exceeds the kernel's buffers.
     const int* geo;
     int* geo_bad;
+    // Ragged batches run their classes' kernels at once (programmatic
+    // dependent launches in one stream).  kTrigger: the next class's kernel
+    // may start as soon as this one's CTAs have; kJoin: the last CTA of this
+    // kernel to finish (counted in *done, zeroed before the launch) waits for
+    // the kernel before, so that the last kernel's end is the end of all.
+    enum { kTrigger = 1, kJoin = 2 };
+    int overlap;
+    int* done;
 };
+
+// The two ends of a class's kernel in a ragged batch (see FusedArgs::overlap),
+// called by every thread of every CTA.
+__device__ __forceinline__ void class_begin(const FusedArgs& a) {
+    if (a.overlap & FusedArgs::kTrigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void class_end(const FusedArgs& a) {
+    if (!(a.overlap & FusedArgs::kJoin)) return;
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(a.done, 1) == (int)gridDim.x - 1)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Launch attribute of a kernel that may start before the one ahead of it in
+// the stream has ended.
+inline void overlap_attribute(cudaLaunchAttribute* attr, const FusedArgs& a) {
+    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr->val.programmaticStreamSerializationAllowed = (a.overlap & FusedArgs::kJoin) ? 1 : 0;
+}
 
 // Default number of cycles a CTA waits for the first part of a cut candidate
 // before giving up (about 2 s at 2 GHz; the schedule leaves the wait a whole
@@ -159,7 +185,8 @@ size_t band_geo_bytes(int n, int nb, int V);   // per-band ray-run records
 // Largest number of clusters of nb CTAs resident at once (cached per device;
 // 0 if the device cannot run them).
 int band_max_clusters(int n, int nb);
-// Launch the record kernel and the cluster kernel with `clusters` clusters.
+// The record kernel, then the cluster kernel with `clusters` clusters.
+int band_prepare(int n, int nb, const FusedArgs& a, cudaStream_t st);
 int band_launch(int n, int nb, const FusedArgs& a, int clusters, cudaStream_t st);
 
 }  // namespace boac
