@@ -60,6 +60,7 @@ struct NvtxPhases {
 // kernels gather and scatter through the checked helpers (count, or -1 if
 // the read failed; reset clears the counter).
 int bounds_faults_fused(int reset);
+int bounds_faults_split(int reset);
 int bounds_faults_bpgroup(int reset);
 int bounds_faults_gradfused(int reset);
 int bounds_faults_grad(int reset);
