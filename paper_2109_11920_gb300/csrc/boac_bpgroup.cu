@@ -22,6 +22,7 @@
 #include "boac_device.cuh"
 #include "boac_internal.h"
 #include "boac_plain_kernels.cuh"
+#include "boac_sched.cuh"
 
 namespace boac {
 
@@ -150,6 +151,134 @@ __global__ void __launch_bounds__(NT) project_group_kernel(int V, float dx, cons
     }
 }
 
+// One MLEM iteration's work on one sample grid of one candidate: q of the
+// grid's views, r = S / q, and the grid's back-projection of r into its slice
+// of `partial`.  A grid's rays belong to it alone, so nothing is exchanged
+// with other CTAs and the steps need no launch each (projection, ratio and
+// back-projection kernels before).  The sums are those of
+// project_group_kernel (four segments per ray, its sample order) and
+// bp_group_kernel, bit for bit: the samples of F go through W, where the
+// threads of a ray's segment add them up in order, one view per half of the
+// CTA; the scatter runs in schedule order.
+template <int N, bool QUAD>
+struct GroupStep {
+    static constexpr int NT = 8 * N, P = N + 1, WP = N + 1;
+    static constexpr int IMG = (N + 1) * (N + 2) + 1 + kScatterPad;
+    static constexpr size_t SMEM = sizeof(float) * ((size_t)IMG + (size_t)N * WP + 16 * N + 4 * N);
+};
+template <int N, bool QUAD>
+__global__ void __launch_bounds__(8 * N, N <= 96 ? 2 : 1)
+    mlem_group_kernel(int V, float dx, const float* __restrict__ tab, const float* __restrict__ S, long long s_stride,
+                      const float* __restrict__ F, const unsigned short* __restrict__ sched,
+                      float* __restrict__ partial) {
+    using G = GroupStep<N, QUAD>;
+    constexpr int NT = G::NT, P = G::P, WP = G::WP, IMG = G::IMG;
+    constexpr int SEG = N / 8;            // gather, weights: samples per thread
+    constexpr int SUM = 4, RUN = N / SUM;  // segments of a ray's sum
+    extern __shared__ __align__(16) float smem[];
+    float* img = smem;         // padded F, then the padded accumulator
+    float* W = img + IMG;      // [N][WP] samples of F, then weights
+    float* red = W + N * WP;   // [4][SUM][N] segment sums
+    float* rr = red + 16 * N;  // [4][N] r per view, at the view's bin
+    const int gi = blockIdx.x, cand = blockIdx.y, ngrid = QUAD ? V / 4 : V / 2;
+    const int tid = threadIdx.x, lb = tid % N, k0 = tid / N * SEG;
+    const size_t nn = (size_t)N * N;
+    const float* tb = tab + (size_t)cand * V * nn;
+    const float* f = F + (size_t)cand * nn;
+    const float* Sc = S + (size_t)cand * s_stride;
+    const unsigned short* gs = sched + (size_t)gi * 9 * SchedShape<N>::CLS_ENTRIES;
+    for (int i = tid; i < IMG; i += NT) img[i] = 0.0f;
+    __syncthreads();
+    for (int i = tid; i < (int)nn; i += NT) img[(i / N + 1) * P + (i % N) + 1] = __ldg(f + i);
+    float cs, sn;
+    view_cos_sin(gi, V, &cs, &sn);
+    const float c = 0.5f * (float)(N - 1);
+    __syncthreads();
+    {
+        ColumnWalk walk(k0, lb, cs, sn, c);
+#pragma unroll 4
+        for (int s = 0; s < SEG; ++s) W[(k0 + s) * WP + lb] = bilerp_pos<N, P>(img, walk.next());
+    }
+    __syncthreads();
+    for (int i = tid; i < IMG; i += NT) img[i] = 0.0f;  // F sampled: now the accumulator
+    // view v, sample (k, b) of the grid in the table: phi (k, b), phi + pi
+    // (n-1-k, n-1-b), phi + pi/2 (n-1-b, k), phi + 3pi/2 (b, n-1-k)
+    const int views[4] = {gi, gi + V / 2, gi + V / 4, gi + 3 * V / 4};
+    const float* t1 = tb + (size_t)views[0] * nn;
+    const float* t2 = tb + (size_t)views[1] * nn;
+    const float* t3 = tb + (size_t)views[2] * nn;
+    const float* t4 = tb + (size_t)views[3] * nn;
+    {
+        const int half = tid / (SUM * N), seg = tid / N % SUM, r0 = seg * RUN;
+        const float* t = half ? t2 + (N - 1 - lb) + (size_t)(N - 1 - r0) * N : t1 + lb + (size_t)r0 * N;
+        const int step = half ? -N : N;
+        float a = 0.0f;
+#pragma unroll 8
+        for (int s = 0; s < RUN; ++s) a = fmaf(__ldg(t + s * step), W[(r0 + s) * WP + lb], a);
+        red[(half * SUM + seg) * N + lb] = a;
+        if (QUAD) {
+            const float* u = half ? t4 + (N - 1 - lb) + (size_t)r0 * N : t3 + lb + (size_t)(N - 1 - r0) * N;
+            a = 0.0f;
+#pragma unroll 8
+            for (int s = 0; s < RUN; ++s) a = fmaf(__ldg(u - s * step), W[lb * WP + r0 + s], a);
+            red[((2 + half) * SUM + seg) * N + lb] = a;
+        }
+    }
+    __syncthreads();
+    for (int t = tid; t < (QUAD ? 4 : 2) * N; t += NT) {
+        const int vi = t / N, j = t % N, bin = (vi & 1) ? N - 1 - j : j;
+        float sum = 0.0f;
+#pragma unroll
+        for (int s2 = 0; s2 < SUM; ++s2) sum += red[(vi * SUM + s2) * N + j];
+        const float q = dx * sum;
+        rr[vi * N + bin] = q > 0.0f ? __ldg(Sc + (size_t)views[vi] * N + bin) / q : 0.0f;
+    }
+    __syncthreads();
+    SchedSlots<N, NT> sched0;
+    sched0.load(gs);
+    {
+        const float y1 = rr[lb], y2 = rr[N + (N - 1 - lb)];
+#pragma unroll 4
+        for (int s = 0; s < SEG; ++s) {
+            const int k = k0 + s;
+            W[k * WP + lb] = dx * fmaf(__ldg(t1 + (size_t)k * N + lb), y1,
+                                       __ldg(t2 + (size_t)(N - 1 - k) * N + (N - 1 - lb)) * y2);
+        }
+    }
+    if (QUAD) {
+        __syncthreads();
+        const int k = lb;
+        const float y3 = rr[2 * N + k], y4 = rr[3 * N + (N - 1 - k)];
+#pragma unroll 4
+        for (int s = 0; s < SEG; ++s) {
+            const int b = k0 + s;
+            W[k * WP + b] += dx * fmaf(__ldg(t3 + (size_t)(N - 1 - b) * N + k), y3,
+                                       __ldg(t4 + (size_t)b * N + (N - 1 - k)) * y4);
+        }
+    }
+    __syncthreads();
+    scatter_scheduled<N, NT, P, WP, true>(W, img, cs, sn, c, gs, sched0);
+    float* out = partial + ((size_t)cand * ngrid + gi) * nn;
+    for (int i = tid; i < (int)nn; i += NT) out[i] = img[(i / N + 1) * P + (i % N) + 1];
+}
+
+// The iteration's end: z = sum over grids of partial, in grid order, and
+// F <- F z / sens (0 where sens = 0).
+__global__ void sum_update_kernel(int B, int ngrid, int nn, const float* __restrict__ partial,
+                                  const float* __restrict__ sens, float* __restrict__ F) {
+    const long long total = (long long)B * nn;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long cand = i / nn, pix = i % nn;
+        const float* p = partial + cand * ngrid * (long long)nn + pix;
+        float s = 0.0f;
+#pragma unroll 8
+        for (int g = 0; g < ngrid; ++g) s += __ldcg(p + (long long)g * nn);
+        const float sv = sens[i];
+        F[i] = sv > 0.0f ? F[i] * s / sv : 0.0f;
+    }
+}
+
 // out[cand][pix] (+)= sum over grids of partial[cand][grid][pix], grid order.
 __global__ void sum_grids_kernel(int B, int ngrid, int nn, const float* __restrict__ partial,
                                  float* __restrict__ out, int accumulate) {
@@ -217,9 +346,7 @@ int backproject_table(const boac_geom* g, int B, const float* tab, const float* 
                       int accumulate, float* partial, cudaStream_t st) {
     const int n = g->n, V = g->n_views;
     if (!bp_grouped(g) || !partial) {
-        const dim3 pg((unsigned)(((size_t)n * n + kPixThreads - 1) / kPixThreads), B);
-        backproject_gather_kernel<<<pg, kPixThreads, sizeof(float) * 2 * V, st>>>(n, V, scale, tab, y, out,
-                                                                                 accumulate);
+        backproject_gather(n, V, B, scale, tab, y, out, accumulate, st);
         return launch_status();
     }
     const bool quad = V % 4 == 0;
@@ -253,6 +380,52 @@ int project_table(const boac_geom* g, int B, const float* tab, const float* F, f
     X(64, 256) X(96, 384) X(128, 512)
 #undef X
     return s;
+}
+
+template <int N, bool QUAD>
+static int mlem_group_launch(int V, int B, float dx, const float* tab, const float* S, long long s_stride,
+                             const float* F, const unsigned short* sched, float* partial, cudaStream_t st) {
+    constexpr size_t smem = GroupStep<N, QUAD>::SMEM;
+    constexpr int kDev = 64;
+    static bool attr_set[kDev];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDev) return launch_status();
+    if (!attr_set[dev]) {
+        if (cudaFuncSetAttribute(mlem_group_kernel<N, QUAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem) != cudaSuccess)
+            return launch_status();
+        attr_set[dev] = true;
+    }
+    mlem_group_kernel<N, QUAD><<<dim3(QUAD ? V / 4 : V / 2, B), 8 * N, smem, st>>>(V, dx, tab, S, s_stride, F, sched,
+                                                                                 partial);
+    return launch_status();
+}
+
+bool mlem_grouped(const boac_geom* g) { return bp_grouped(g); }
+
+size_t mlem_group_sched_bytes(const boac_geom* g) {
+    return bp_grouped(g) ? sched_bytes(g->n, g->n_views % 4 == 0 ? g->n_views / 4 : g->n_views / 2) : 0;
+}
+
+const unsigned short* mlem_group_sched(const boac_geom* g, unsigned short* ws, cudaStream_t st, int* status) {
+    const int V = g->n_views;
+    return sched_prepare(g->n, V, V % 4 == 0 ? V / 4 : V / 2, g->n + 1 /* GroupStep<N>::WP */, ws, st, status);
+}
+
+int mlem_group_iteration(const boac_geom* g, int B, float dx, const float* tab, const float* S, long long s_stride,
+                         float* F, const float* sens, const unsigned short* sched, float* partial, cudaStream_t st) {
+    const int n = g->n, V = g->n_views;
+    const bool quad = V % 4 == 0;
+    int s = BOAC_EUNSUPPORTED;
+#define X(NV)                                                                                      \
+    if (n == NV)                                                                                   \
+        s = quad ? mlem_group_launch<NV, true>(V, B, dx, tab, S, s_stride, F, sched, partial, st)  \
+                 : mlem_group_launch<NV, false>(V, B, dx, tab, S, s_stride, F, sched, partial, st);
+    X(64) X(96) X(128)
+#undef X
+    if (s != BOAC_OK) return s;
+    sum_update_kernel<<<grid_1d((long long)B * n * n, 128), 128, 0, st>>>(B, quad ? V / 4 : V / 2, n * n, partial, sens, F);
+    return launch_status();
 }
 
 #ifdef BOAC_CHECKED

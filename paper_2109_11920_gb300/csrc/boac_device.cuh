@@ -156,15 +156,34 @@ struct ColumnWalk {
     }
 };
 
+// The bilinear sample, and its transpose (g times each weight added), of the
+// footprint at p with fractions frac, as bilerp_padded and scatter_padded
+// compute them.
+template <int P>
+__device__ __forceinline__ float bilerp_cell(const float* p, float2 frac) {
+    const float2 v0 = make_float2(p[0], p[P]), v1 = make_float2(p[1], p[P + 1]);
+    const float2 tb = __ffma2_rn(pair(frac.x), sub2(v1, v0), v0);  // (top, bottom)
+    return fmaf(frac.y, tb.y - tb.x, tb.x);
+}
+template <int P>
+__device__ __forceinline__ void scatter_cell(float* p, float2 frac, float g) {
+    const float g1 = __fmul_rn(g, frac.y);
+    const float2 row = make_float2(__fsub_rn(g, g1), g1);  // weights of the footprint's rows
+    const float2 au = pair(frac.x);
+    const float2 left = __fadd2_rn(make_float2(p[0], p[P]), sub2_mul(row, row, au));
+    const float2 right = __ffma2_rn(row, au, make_float2(p[1], p[P + 1]));
+    p[0] = left.x;
+    p[1] = right.x;
+    p[P] = left.y;
+    p[P + 1] = right.y;
+}
+
 // bilerp_padded at a position.
 template <int N, int P>
 __device__ __forceinline__ float bilerp_pos(const float* img, float2 pos) {
     const Cell<N, P> x(pos);
     if (!x.in || !index_ok(x.cell, (long long)P * (N + 1))) return 0.0f;
-    const float* p = img + x.cell;
-    const float2 v0 = make_float2(p[0], p[P]), v1 = make_float2(p[1], p[P + 1]);
-    const float2 tb = __ffma2_rn(pair(x.frac.x), sub2(v1, v0), v0);  // (top, bottom)
-    return fmaf(x.frac.y, tb.y - tb.x, tb.x);
+    return bilerp_cell<P>(img + x.cell, x.frac);
 }
 
 // Transpose of bilerp_padded: add g times each bilinear weight to the four

@@ -561,7 +561,7 @@ static int score_grad_run(const boac_geom* g, const boac_tissue* t, const float*
     const double* lgS = include_lgamma && s_stride == 0
                             ? lgamma_sum((int)vb, S, reinterpret_cast<double*>(base + lay.lg), st)
                             : nullptr;
-    loglik_kernel<<<B, 256, 0, st>>>((int)vb, qK, S, s_stride, include_lgamma, L, lgS);
+    loglik_launch((int)vb, B, qK, S, s_stride, include_lgamma, L, lgS, nullptr, st);
     if (F_out) cudaMemcpyAsync(F_out, Fk, sizeof(float) * cnt_pix, cudaMemcpyDeviceToDevice, st);
     qbar_final_kernel<<<g1b, 256, 0, st>>>(B, (int)vb, S, s_stride, qK, qbar);
     backproject_table(g, B, tab, qbar, dx, Fbar, 0, partial, st);

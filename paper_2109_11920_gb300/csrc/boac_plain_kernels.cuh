@@ -18,9 +18,9 @@ __global__ void project_otf_kernel(int n, int V, float dx, const float* __restri
                                    const float* __restrict__ F, float* __restrict__ q);
 __global__ void project_table_kernel(int n, int V, float dx, const float* __restrict__ tab,
                                      const float* __restrict__ F, float* __restrict__ q);
-__global__ void backproject_gather_kernel(int n, int V, float scale, const float* __restrict__ tab,
-                                          const float* __restrict__ y, float* __restrict__ out,
-                                          int accumulate);
+// out[cand] (+)= scale sum_v B_v^T (tab_v y_v), per-pixel gather (boac_plain.cu).
+void backproject_gather(int n, int V, int B, float scale, const float* tab, const float* y, float* out,
+                        int accumulate, cudaStream_t st);
 __global__ void ratio_kernel(int count, const float* __restrict__ S, const float* __restrict__ q,
                              float* __restrict__ r);
 __global__ void update_kernel(int count, float* __restrict__ F, const float* __restrict__ bp,
@@ -30,6 +30,9 @@ __global__ void update_kernel(int count, float* __restrict__ F, const float* __r
 __global__ void loglik_kernel(int nbin, const float* __restrict__ q, const float* __restrict__ S,
                               long long s_stride, int include_lgamma, double* __restrict__ L,
                               const double* __restrict__ lgS, int* status = nullptr);
+// Launch it for B candidates, on clusters where that is faster (same bits).
+int loglik_launch(int nbin, int B, const float* q, const float* S, long long s_stride, int include_lgamma, double* L,
+                  const double* lgS, int* status, cudaStream_t st);
 // sum_i lgamma(S_i + 1) of one sinogram S[nbin] into scratch[0]
 // (scratch: kLgammaScratchDoubles doubles, 8-byte aligned); returns scratch.
 constexpr int kLgammaScratchDoubles = 31;
@@ -52,6 +55,14 @@ size_t bp_partial_floats(const boac_geom* g, int B);
 // F in shared memory, or one thread per ray where no grouped kernel exists.
 int project_table(const boac_geom* g, int B, const float* tab, const float* F, float dx, float* q,
                   cudaStream_t st);
+// One whole MLEM iteration F <- F A^T(S / A F) / sens from the table, for
+// geometries with grouped kernels (mlem_grouped): two launches, `partial` as
+// above, sched from mlem_group_sched (ws: mlem_group_sched_bytes of scratch).
+bool mlem_grouped(const boac_geom* g);
+size_t mlem_group_sched_bytes(const boac_geom* g);
+const unsigned short* mlem_group_sched(const boac_geom* g, unsigned short* ws, cudaStream_t st, int* status);
+int mlem_group_iteration(const boac_geom* g, int B, float dx, const float* tab, const float* S, long long s_stride,
+                         float* F, const float* sens, const unsigned short* sched, float* partial, cudaStream_t st);
 int backproject_table(const boac_geom* g, int B, const float* tab, const float* y, float scale, float* out,
                       int accumulate, float* partial, cudaStream_t st);
 

@@ -299,16 +299,7 @@ __device__ __forceinline__ void scatter_scheduled(const float* __restrict__ W, f
             ok = ok && index_ok(wi, (long long)N * WP) && index_ok(x.cell, (long long)P * (N + 1));
             float g = 0.0f;
             if (ok) g = W[wi];
-            float* p = img1 + (ok ? x.cell : pad_cell);
-            const float g1 = __fmul_rn(g, x.frac.y);
-            const float2 row = make_float2(__fsub_rn(g, g1), g1);  // weights of the footprint's rows
-            const float2 au = pair(x.frac.x);
-            const float2 left = __fadd2_rn(make_float2(p[0], p[P]), sub2_mul(row, row, au));
-            const float2 right = __ffma2_rn(row, au, make_float2(p[1], p[P + 1]));
-            p[0] = left.x;
-            p[1] = right.x;
-            p[P] = left.y;
-            p[P + 1] = right.y;
+            scatter_cell<P>(img1 + (ok ? x.cell : pad_cell), x.frac, g);
         }
         __syncthreads();
         cur = nxt;

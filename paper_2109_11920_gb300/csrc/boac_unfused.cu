@@ -16,7 +16,7 @@ namespace boac {
 namespace {
 
 struct UnfusedLayout {
-    size_t status, tab, sens, z, q, r, partial, total;
+    size_t status, tab, sens, z, q, r, partial, sched, total;
 };
 
 UnfusedLayout unfused_layout(const boac_geom* g, int B) {
@@ -35,6 +35,7 @@ UnfusedLayout unfused_layout(const boac_geom* g, int B) {
     l.q = take(Bs * vb);
     l.r = take(Bs * vb);
     l.partial = take(bp_partial_floats(g, B));
+    l.sched = take(mlem_group_sched_bytes(g) / sizeof(float));
     l.total = off;
     return l;
 }
@@ -62,8 +63,18 @@ int mlem_unfused(const boac_geom* g, const float* mu, const float* S, long long 
     attenuation_table_kernel<<<ray_grid(g, B), kRayThreads, 0, st>>>(g->n, g->n_views, dx, mu, tab);
     int s = backproject_table(g, B, tab, nullptr, dx, sens, 0, partial, st);
     if (s != BOAC_OK) return s;
+    const unsigned short* sched = nullptr;
+    if (K > 0 && mlem_grouped(g)) {
+        sched = mlem_group_sched(g, reinterpret_cast<unsigned short*>(base + l.sched), st, &s);
+        if (s != BOAC_OK) return s;
+    }
     for (int it = 0; it < K; ++it) {
         BOAC_RANGE("MLEM iteration");
+        if (sched) {
+            s = mlem_group_iteration(g, B, dx, tab, S, s_stride, F, sens, sched, partial, st);
+            if (s != BOAC_OK) return s;
+            continue;
+        }
         s = project_table(g, B, tab, F, dx, q, st);
         if (s != BOAC_OK) return s;
         ratio_batched_kernel<<<grid_1d(cnt_bin, 256), 256, 0, st>>>(B, (int)vb, S, s_stride, q, r);
@@ -79,8 +90,9 @@ int mlem_unfused(const boac_geom* g, const float* mu, const float* S, long long 
         const double* lgS = include_lgamma && s_stride == 0
                                 ? lgamma_sum((int)vb, S, reinterpret_cast<double*>(base + l.status + 8), st)
                                 : nullptr;
-        loglik_kernel<<<B, 256, 0, st>>>((int)vb, q, S, s_stride, include_lgamma, L, lgS,
-                                         reinterpret_cast<int*>(base + l.status));
+        s = loglik_launch((int)vb, B, q, S, s_stride, include_lgamma, L, lgS, reinterpret_cast<int*>(base + l.status),
+                          st);
+        if (s != BOAC_OK) return s;
     }
     return launch_status();
 }
