@@ -21,6 +21,7 @@
 
 #include "boac_device.cuh"
 #include "boac_internal.h"
+#include "boac_ops.h"
 #include "boac_plain_kernels.cuh"
 #include "boac_sched.cuh"
 
@@ -398,6 +399,11 @@ static int mlem_group_launch(int V, int B, float dx, const float* tab, const flo
     }
     mlem_group_kernel<N, QUAD><<<dim3(QUAD ? V / 4 : V / 2, B), 8 * N, smem, st>>>(V, dx, tab, S, s_stride, F, sched,
                                                                                  partial);
+    return launch_status();
+}
+
+int sum_partial_images(int B, int shares, int nn, const float* partial, float* out, cudaStream_t st) {
+    sum_grids_kernel<<<grid_1d((long long)B * nn, 256), 256, 0, st>>>(B, shares, nn, partial, out, 0);
     return launch_status();
 }
 

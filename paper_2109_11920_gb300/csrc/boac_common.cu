@@ -76,7 +76,8 @@ extern "C" int boac_bounds_faults(int* faults, int reset) {
 #ifdef BOAC_CHECKED
     if (!faults) return BOAC_EINVAL;
     // one counter per translation unit that uses the checked helpers
-    int (*const readers[])(int) = {bounds_faults_fused,   bounds_faults_split,   bounds_faults_bpgroup, bounds_faults_gradfused,
+    int (*const readers[])(int) = {bounds_faults_fused,   bounds_faults_split,   bounds_faults_ops,
+                                   bounds_faults_bpgroup, bounds_faults_gradfused,
                                    bounds_faults_grad,    bounds_faults_plain,   bounds_faults_unfused,
                                    bounds_faults_sysmat,  bounds_faults_band,    bounds_faults_raster};
     int total = 0;

@@ -61,6 +61,7 @@ struct NvtxPhases {
 // the read failed; reset clears the counter).
 int bounds_faults_fused(int reset);
 int bounds_faults_split(int reset);
+int bounds_faults_ops(int reset);
 int bounds_faults_bpgroup(int reset);
 int bounds_faults_gradfused(int reset);
 int bounds_faults_grad(int reset);

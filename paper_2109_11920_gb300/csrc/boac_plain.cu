@@ -15,6 +15,7 @@
 
 #include "boac_device.cuh"
 #include "boac_internal.h"
+#include "boac_ops.h"
 #include "boac_plain_kernels.cuh"
 
 namespace cg = cooperative_groups;
@@ -377,6 +378,7 @@ extern "C" int boac_project(const boac_geom* g, const float* mu, const float* F,
                             void* stream) {
     BOAC_RANGE("boac_project");
     if (!geom_ok(g) || !mu || !F || !q || B < 1 || B > 65535) return BOAC_EINVAL;
+    if (ops_on_grids(g)) return project_on_grids(g, mu, F, B, q, as_stream(stream));
     project_otf_kernel<<<ray_grid(g, B), kRayThreads, 0, as_stream(stream)>>>(
         g->n, g->n_views, g->pixel_cm, mu, F, q);
     return launch_status();
@@ -398,6 +400,12 @@ extern "C" int boac_backproject(const boac_geom* g, const float* mu, const float
         base + align256(sizeof(float) * (size_t)chunk * g->n_views * nn));
     for (int c0 = 0; c0 < B; c0 += chunk) {
         const int cb = (B - c0) < chunk ? (B - c0) : chunk;
+        if (ops_on_grids(g)) {  // no table: its room holds the schedule if the cache has none
+            const int s = backproject_on_grids(g, mu + c0 * nn, y ? y + (size_t)c0 * g->n_views * g->n_bins : nullptr, cb,
+                                               out + c0 * nn, partial, reinterpret_cast<unsigned short*>(base), st);
+            if (s != BOAC_OK) return s;
+            continue;
+        }
         attenuation_table_kernel<<<ray_grid(g, cb), kRayThreads, 0, st>>>(
             g->n, g->n_views, g->pixel_cm, mu + c0 * nn, tab);
         int s = launch_status();
@@ -426,7 +434,8 @@ extern "C" int boac_score(const boac_geom* g, const float* mu, const float* S, l
     const size_t vb = (size_t)g->n_views * g->n_bins;
     if (!ws || ws_bytes < sizeof(float) * vb * B) return BOAC_EWORKSPACE;
     float* q = static_cast<float*>(ws);
-    int s = boac_project(g, mu, F, B, q, stream);
+    project_otf_kernel<<<ray_grid(g, B), kRayThreads, 0, as_stream(stream)>>>(g->n, g->n_views, g->pixel_cm, mu, F, q);
+    int s = launch_status();
     if (s != BOAC_OK) return s;
     return boac_loglik(g, q, S, s_stride, B, include_lgamma, L, stream);
 }
