@@ -88,6 +88,34 @@ __device__ __forceinline__ void class_end(const FusedArgs& a) {
     if (threadIdx.x == 0 && atomicAdd(a.done, 1) == (int)gridDim.x - 1)
         asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// Element i of every rank's copy of a shared-memory array, summed in rank
+// order; and the same value stored into every rank's copy.  All the loads are
+// in flight at once (one after the other, eight ranks' latencies add up: one
+// gradient at 128 x 128, 20 iterations: 4.32 -> 3.97 ms).
+// (In assembly: the compiler would keep G mapped addresses in registers across
+// the iterations.)
+template <int G>
+__device__ __forceinline__ float rank_sum(const float* a, int i) {
+    const unsigned at = (unsigned)__cvta_generic_to_shared(a + i);
+    float v[G], s = 0.0f;
+#pragma unroll
+    for (int r = 0; r < G; ++r)
+        asm volatile("{\n.reg .u32 t;\nmapa.shared::cluster.u32 t, %1, %2;\nld.shared::cluster.f32 %0, [t];\n}"
+                     : "=f"(v[r])
+                     : "r"(at), "r"(r));
+#pragma unroll
+    for (int r = 0; r < G; ++r) s += v[r];
+    return s;
+}
+template <int G>
+__device__ __forceinline__ void rank_put(float* a, int i, float v) {
+    const unsigned at = (unsigned)__cvta_generic_to_shared(a + i);
+#pragma unroll
+    for (int r = 0; r < G; ++r)
+        asm volatile("{\n.reg .u32 t;\nmapa.shared::cluster.u32 t, %0, %1;\nst.shared::cluster.f32 [t], %2;\n}" ::"r"(at),
+                     "r"(r), "f"(v)
+                     : "memory");
+}
 // Launch attribute of a kernel that may start before the one ahead of it in
 // the stream has ended.
 inline void overlap_attribute(cudaLaunchAttribute* attr, const FusedArgs& a) {

@@ -411,10 +411,7 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
             cl.sync();
             for (int i = tid; i < (R1 - R0) * N; i += NT) {
                 const int pi = (R0 + i / N + 1) * P + (i % N) + 1;
-                float sv = 0.0f;
-#pragma unroll 1
-                for (int r = 0; r < G; ++r) sv += cl.map_shared_rank(img1, r)[pi];
-                sens[i] = sv;
+                sens[i] = rank_sum<G>(img1, pi);
             }
             cl.sync();
             for (int i = tid; i < NN; i += NT) img0[(i / N + 1) * P + (i % N) + 1] = Fc[i];
@@ -609,13 +606,9 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
                 cl.sync();
                 for (int i = tid; i < (R1 - R0) * N; i += NT) {
                     const int pi = (R0 + i / N + 1) * P + (i % N) + 1;
-                    float bp = 0.0f;
-#pragma unroll 1
-                    for (int r = 0; r < G; ++r) bp += cl.map_shared_rank(img1, r)[pi];
                     const float sv = sens[i];
-                    const float fn = sv > 0.0f ? img0[pi] * bp / sv : 0.0f;
-#pragma unroll 1
-                    for (int r = 0; r < G; ++r) cl.map_shared_rank(img0, r)[pi] = fn;
+                    const float bp = rank_sum<G>(img1, pi);
+                    rank_put<G>(img0, pi, sv > 0.0f ? img0[pi] * bp / sv : 0.0f);
                 }
                 cl.sync();
                 for (int i = tid; i < IMG; i += NT) img1[i] = 0.0f;

@@ -127,11 +127,7 @@ __global__ void __launch_bounds__(8 * N, 1) grad_fused_kernel(GradFusedArgs a) {
     // the accumulators of all ranks at padded index pi, summed in rank order
     auto acc_sum = [&](int pi) -> float {
         if constexpr (G > 1) {
-            cg::cluster_group cl = cg::this_cluster();
-            float s = 0.0f;
-#pragma unroll 1
-            for (int r = 0; r < G; ++r) s += cl.map_shared_rank(img1, r)[pi];
-            return s;
+            return rank_sum<G>(img1, pi);
         } else {
             return img1[pi];
         }
@@ -139,9 +135,7 @@ __global__ void __launch_bounds__(8 * N, 1) grad_fused_kernel(GradFusedArgs a) {
     // value v of padded index pi into every rank's img0
     auto put_all = [&](int pi, float v) {
         if constexpr (G > 1) {
-            cg::cluster_group cl = cg::this_cluster();
-#pragma unroll 1
-            for (int r = 0; r < G; ++r) cl.map_shared_rank(img0, r)[pi] = v;
+            rank_put<G>(img0, pi, v);
         } else {
             img0[pi] = v;
         }
