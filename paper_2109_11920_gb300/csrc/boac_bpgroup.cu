@@ -369,7 +369,7 @@ int project_table(const boac_geom* g, int B, const float* tab, const float* F, f
                   cudaStream_t st) {
     const int n = g->n, V = g->n_views;
     if (!bp_grouped(g)) {
-        project_table_kernel<<<ray_grid(g, B), kRayThreads, 0, st>>>(n, V, dx, tab, F, q);
+        project_table_rays(g, B, dx, tab, F, q, st);
         return launch_status();
     }
     const bool quad = V % 4 == 0;

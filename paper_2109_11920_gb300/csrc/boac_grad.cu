@@ -530,7 +530,7 @@ static int score_grad_run(const boac_geom* g, const boac_tissue* t, const float*
     NvtxPhases phase("gradient: forward MLEM with checkpoints");
     int s = rasterize_launch(g, t, c, t ? 6 : kParams, B, BOAC_RASTER_AREA, mu, st);
     if (s != BOAC_OK) return s;
-    attenuation_table_kernel<<<rg, kRayThreads, 0, st>>>(n, V, dx, mu, tab);
+    attenuation_table(g, B, mu, tab, st);
     backproject_table(g, B, tab, nullptr, dx, sens, 0, partial, st);
     cudaMemsetAsync(abar, 0, sizeof(float) * (size_t)B * V * nn, st);
     cudaMemsetAsync(sensbar, 0, sizeof(float) * cnt_pix, st);

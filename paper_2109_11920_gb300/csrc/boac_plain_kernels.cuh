@@ -18,6 +18,11 @@ __global__ void project_otf_kernel(int n, int V, float dx, const float* __restri
                                    const float* __restrict__ F, float* __restrict__ q);
 __global__ void project_table_kernel(int n, int V, float dx, const float* __restrict__ tab,
                                      const float* __restrict__ F, float* __restrict__ q);
+// The same with their images in shared memory where those fit (same bits).
+void attenuation_table(const boac_geom* g, int B, const float* mu, float* tab, cudaStream_t st);
+void project_rays(const boac_geom* g, int B, const float* mu, const float* F, float* q, cudaStream_t st);
+void project_table_rays(const boac_geom* g, int B, float dx, const float* tab, const float* F, float* q,
+                        cudaStream_t st);
 // out[cand] (+)= scale sum_v B_v^T (tab_v y_v), per-pixel gather (boac_plain.cu).
 void backproject_gather(int n, int V, int B, float scale, const float* tab, const float* y, float* out,
                         int accumulate, cudaStream_t st);

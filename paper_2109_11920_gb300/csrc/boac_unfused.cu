@@ -60,7 +60,7 @@ int mlem_unfused(const boac_geom* g, const float* mu, const float* S, long long 
     // the status word boac_workspace_status reads: this path has no waits
     cudaMemsetAsync(base + l.status, 0, sizeof(int), st);
     BOAC_RANGE("set-up: attenuation tables, sensitivity");
-    attenuation_table_kernel<<<ray_grid(g, B), kRayThreads, 0, st>>>(g->n, g->n_views, dx, mu, tab);
+    attenuation_table(g, B, mu, tab, st);
     int s = backproject_table(g, B, tab, nullptr, dx, sens, 0, partial, st);
     if (s != BOAC_OK) return s;
     const unsigned short* sched = nullptr;
