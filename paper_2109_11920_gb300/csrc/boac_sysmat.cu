@@ -281,23 +281,34 @@ __device__ __forceinline__ void fma8(float* acc, const Group8& a, const Group8& 
     acc[7] = fmaf(a.hi.w, b.hi.w, acc[7]);
 }
 
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-    return x;
-}
-
-// The eight warp sums of acc[]; lane c (< 8) returns the sum of acc[c].
+// The eight warp sums of acc[]; lane c (< 8) returns the sum of acc[c].  The
+// sums are those of a butterfly over lane distances 16, 8, 4, 2, 1 for each;
+// at the first three a lane hands on the half of its candidates that it does
+// not keep, so ten exchanges do instead of forty.
 __device__ __forceinline__ float warp_sums8(const float* acc, int lane) {
-    float mine = 0.0f;
+    float x[kCandGroup];
 #pragma unroll
-    for (int cc = 0; cc < kCandGroup; ++cc) {
-        const float s = warp_sum(acc[cc]);
-        if (cc == lane) mine = s;
+    for (int cc = 0; cc < kCandGroup; ++cc) x[cc] = acc[cc];
+#pragma unroll
+    for (int step = 0; step < 3; ++step) {
+        const int off = 16 >> step, half = 4 >> step;
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const float give = up ? x[i] : x[i + half], keep = up ? x[i + half] : x[i];
+            x[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
     }
-    return mine;
+    float s = x[0];
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    // candidate c ended in the lanes whose bits 4, 3, 2 are c's bits 2, 1, 0
+    return __shfl_sync(0xffffffffu, s, (lane & 7) << 2);
 }
 
+// Entries of a lane in flight in the two products (their index, value and
+// operand loads); 1, 4 and 8 are 1 to 3 % slower, 32-byte vector loads 7 %.
+constexpr int kProductUnroll = 2;
 constexpr int kFillWarps = 4;  // value fill: one warp per row, a group of candidates
 
 // Values of the candidate group blockIdx.y: one warp per row.  For each
@@ -310,7 +321,7 @@ __global__ void __launch_bounds__(kFillWarps * 32)
 values_kernel(int n, int V, float dx, int R, long long nnz, int B, const int* __restrict__ row_ptr,
               const int* __restrict__ col, const int* __restrict__ contrib, const int* __restrict__ posT,
               const float* __restrict__ mu, float* __restrict__ vals) {
-    __shared__ float sh_a[kFillWarps][kCandGroup][kMaxN];
+    __shared__ __align__(16) float sh_a[kFillWarps][kMaxN][kCandGroup];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = blockIdx.x * kFillWarps + warp, grp = blockIdx.y;
     if (row >= R) return;  // whole warps leave; only warp-level synchronisation follows
@@ -322,9 +333,9 @@ values_kernel(int n, int V, float dx, int R, long long nnz, int B, const int* __
     const int k_lo = lane * per;
     for (int cc = 0; cc < kCandGroup; ++cc) {
         const int cand = grp * kCandGroup + cc;
-        float* a = sh_a[warp][cc];
+        float(*a)[kCandGroup] = sh_a[warp];  // a sample's candidates side by side: 16-byte reads below
         if (cand >= B) {
-            for (int k = lane; k < n; k += 32) a[k] = 0.0f;
+            for (int k = lane; k < n; k += 32) a[k][cc] = 0.0f;
             continue;
         }
         const float* m_img = mu + (size_t)cand * n * n;
@@ -353,7 +364,7 @@ values_kernel(int n, int V, float dx, int R, long long nnz, int B, const int* __
         for (int q = kMaxN / 32 - 1; q >= 0; --q) {
             const int k = k_lo + q;
             if (q < per && k < n) {
-                a[k] = expf(-dx * (0.5f * m_loc[q] + suffix));
+                a[k][cc] = expf(-dx * (0.5f * m_loc[q] + suffix));
                 suffix += m_loc[q];
             }
         }
@@ -372,8 +383,9 @@ values_kernel(int n, int V, float dx, int R, long long nnz, int B, const int* __
             float u, w;
             sample_uw(k, b, cs, sn, c, &u, &w);
             const float wt = pixel_weight(u, w, i, j, n);
-#pragma unroll
-            for (int cc = 0; cc < kCandGroup; ++cc) acc[cc] = fmaf(sh_a[warp][cc][k], wt, acc[cc]);
+            const float4 a0 = *reinterpret_cast<const float4*>(sh_a[warp][k]);
+            const float4 a1 = *reinterpret_cast<const float4*>(sh_a[warp][k] + 4);
+            fma8(acc, Group8{a0, a1}, Group8{make_float4(wt, wt, wt, wt), make_float4(wt, wt, wt, wt)});
         }
         const float4 lo = make_float4(dx * acc[0], dx * acc[1], dx * acc[2], dx * acc[3]);
         const float4 hi = make_float4(dx * acc[4], dx * acc[5], dx * acc[6], dx * acc[7]);
@@ -442,6 +454,7 @@ forward_kernel(int R, int nn, long long nnz, const int* __restrict__ row_ptr, co
 #pragma unroll
     for (int cc = 0; cc < kCandGroup; ++cc) acc[cc] = 0.0f;
     const int e1 = row_ptr[row + 1];
+#pragma unroll kProductUnroll
     for (int e = row_ptr[row] + lane; e < e1; e += 32) {
         const int p = __ldg(col + e);
         const Group8 v = load8_stream(vA + (size_t)e * kCandGroup);
@@ -481,6 +494,7 @@ backward_update_kernel(int nn, int R, long long nnz, const int* __restrict__ col
 #pragma unroll
     for (int cc = 0; cc < kCandGroup; ++cc) acc[cc] = 0.0f;
     const int e1 = colT_ptr[p + 1];
+#pragma unroll kProductUnroll
     for (int e = colT_ptr[p] + lane; e < e1; e += 32) {
         const int row = __ldg(rowT + e);
         fma8(acc, load8_stream(vT + (size_t)e * kCandGroup), load8(rg + (size_t)row * kCandGroup));
