@@ -374,8 +374,9 @@ static int launch_uniform(const boac_geom* g, const FusedVariant* v, int slots, 
     const long long per = K > 0 ? K : 1, units = (long long)B * per;
     a.cap = split_cap(units, per, slots);
     const int grid = (int)((units + a.cap - 1) / a.cap);
+    // (cluster mode takes whole candidates: no hand-over flags)
     if (cudaMemsetAsync(ws + l.status, 0, sizeof(int), st) != cudaSuccess ||
-        cudaMemsetAsync(ws + l.ready, 0, sizeof(int) * (size_t)B, st) != cudaSuccess)
+        (v->g == 1 && cudaMemsetAsync(ws + l.ready, 0, sizeof(int) * (size_t)B, st) != cudaSuccess))
         return launch_status();
     // one shared sinogram: its ln S! sum once, in the status slot's spare bytes
     if (L && include_lgamma && s_stride == 0) {

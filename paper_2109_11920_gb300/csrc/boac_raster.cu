@@ -120,7 +120,10 @@ int pixel_geom_launch(int n, double dx, double* pg, cudaStream_t st) {
 int rasterize_launch(const boac_geom* g, const boac_tissue* t, const float* p, int pstride, int B,
                      int mode, float* mu, cudaStream_t st) {
     long long total = (long long)((B + kRasterGroup - 1) / kRasterGroup) * g->n * g->n;
-    int threads = 256;
+    // An SM's float64 rate bounds this kernel (a square root and five divisions
+    // per pixel): small batches in small blocks, so that they reach every SM
+    // (one 64 x 64 candidate: 16 blocks of 256 threads took 7 us more).
+    int threads = total >= 256LL * 2 * (sm_count() > 0 ? sm_count() : 1) ? 256 : 64;
     long long blocks = (total + threads - 1) / threads;
     long long cap = 64LL * (sm_count() > 0 ? sm_count() : 1);
     if (blocks > cap) blocks = cap;
