@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(N) band_records_kernel(int V, int* geo, int* b
         s_bad = 0;
     }
     float cs, sn;
-    view_cos_sin(band_base_view(gi, V), V, &cs, &sn);
+    cta_view_cos_sin(band_base_view(gi, V), V, &cs, &sn);
     const float c = 0.5f * (float)(N - 1);
     int lo = -1, hi = -1, cnt = 0;
     for (int k = 0; k < N; ++k) {

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(NT, 1)
     const float* tb = tab + (size_t)cand * V * nn;
     const float* yc = y ? y + (size_t)cand * V * N : nullptr;
     float cs, sn;
-    view_cos_sin(gi, V, &cs, &sn);
+    cta_view_cos_sin(gi, V, &cs, &sn);
     const float c = 0.5f * (float)(N - 1);
     for (int i = tid; i < IMG; i += NT) acc[i] = 0.0f;
     // views phi (sample (k, b)) and phi + pi (its sample (n-1-k, n-1-b)):
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(NT) project_group_kernel(int V, float dx, cons
     for (int i = tid; i < (int)nn; i += NT) img[(i / N + 1) * P + (i % N) + 1] = __ldg(f + i);
     __syncthreads();
     float cs, sn;
-    view_cos_sin(gi, V, &cs, &sn);
+    cta_view_cos_sin(gi, V, &cs, &sn);
     const float c = 0.5f * (float)(N - 1);
     const int v1 = gi, v2 = gi + V / 2, v3 = gi + V / 4, v4 = gi + 3 * V / 4;
     {
@@ -190,9 +190,10 @@ __global__ void __launch_bounds__(8 * N, N <= 96 ? 2 : 1)
     const unsigned short* gs = sched + (size_t)gi * 9 * SchedShape<N>::CLS_ENTRIES;
     for (int i = tid; i < IMG; i += NT) img[i] = 0.0f;
     __syncthreads();
+#pragma unroll 4
     for (int i = tid; i < (int)nn; i += NT) img[(i / N + 1) * P + (i % N) + 1] = __ldg(f + i);
     float cs, sn;
-    view_cos_sin(gi, V, &cs, &sn);
+    cta_view_cos_sin(gi, V, &cs, &sn);
     const float c = 0.5f * (float)(N - 1);
     __syncthreads();
     {

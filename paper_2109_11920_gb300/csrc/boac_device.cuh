@@ -62,6 +62,17 @@ __device__ __forceinline__ void view_cos_sin(int v, int V, float* cs, float* sn)
     }
 }
 
+// view_cos_sin for a whole CTA: one thread evaluates it.  An SM does two
+// float64 operations a cycle, so a float64 sine and cosine by each of 1024
+// threads take 20 us.  Called by all threads; contains a barrier.
+__device__ __forceinline__ void cta_view_cos_sin(int v, int V, float* cs, float* sn) {
+    __shared__ float value[2];
+    if (threadIdx.x == 0) view_cos_sin(v, V, &value[0], &value[1]);
+    __syncthreads();
+    *cs = value[0];
+    *sn = value[1];
+}
+
 // Continuous (column u, row w) pixel index of ray sample k of bin b in the
 // view with (cs, sn): p = s (cs, sn) + t (-sn, cs), s = (b - c) dx,
 // t = (k - c) dx, c = (n - 1) / 2 (bins and samples share the pixel pitch).

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(NT) abar_grid_kernel(int V, float dx, const fl
     const float* x1 = X1 + cand * nn;
     const float* x2 = X2 ? X2 + cand * nn : nullptr;
     float cs, sn;
-    view_cos_sin(gi, V, &cs, &sn);
+    cta_view_cos_sin(gi, V, &cs, &sn);
     const float c = 0.5f * (float)(N - 1);
     auto wt = [&](const float* y, int v, int bin) {
         return dx * (y ? __ldg(y + cand * vb + (size_t)v * N + bin) : 1.0f);

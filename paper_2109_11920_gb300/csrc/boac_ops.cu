@@ -7,8 +7,8 @@
 // once per view through L1 with 128 dependent steps, and the table-based
 // back-projector writes and reads every attenuation factor (8 MB per candidate
 // at 128 x 128 and 120 views); other sizes still use them (boac_plain.cu).
-// Measured, 64 candidates at 128 x 128 and 120 views: projection 272 us
-// (855), back-projection 311 us (790).
+// Measured, 64 candidates at 128 x 128 and 120 views: projection 118 us
+// (855), back-projection 156 us (790).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -73,6 +73,7 @@ __device__ __forceinline__ void run_factors(const float (&m)[SEG], float before,
 
 template <int N, int NT, int P>
 __device__ __forceinline__ void load_image(float* img, const float* __restrict__ src) {
+#pragma unroll 4
     for (int i = threadIdx.x; i < N * N; i += NT) img[(i / N + 1) * P + (i % N) + 1] = __ldg(src + i);
 }
 
@@ -95,14 +96,15 @@ __global__ void __launch_bounds__(8 * N, 1)
     const int g0 = (int)((long long)blockIdx.x * ngrid / gridDim.x);
     const int g1 = (int)((long long)(blockIdx.x + 1) * ngrid / gridDim.x);
     const float c = 0.5f * (float)(N - 1), ndl = -dx * 1.44269504088896340736f;
+    __shared__ float csn[kMaxViews];  // the share's grids (at most half the views)
+    for (int gi = g0 + tid; gi < g1; gi += NT) view_cos_sin(gi, V, &csn[2 * (gi - g0)], &csn[2 * (gi - g0) + 1]);
     for (int i = tid; i < 2 * IMG; i += NT) smem[i] = 0.0f;
     __syncthreads();
     load_image<N, NT, P>(img0, F + (size_t)cand * N * N);
     load_image<N, NT, P>(img1, mu + (size_t)cand * N * N);
     __syncthreads();
     for (int gi = g0; gi < g1; ++gi) {
-        float cs, sn;
-        view_cos_sin(gi, V, &cs, &sn);
+        const float cs = csn[2 * (gi - g0)], sn = csn[2 * (gi - g0) + 1];
         float f[SEG], e[2 * SEG];
         {
             float m[SEG], sum = 0.0f;
@@ -198,13 +200,14 @@ __global__ void __launch_bounds__(8 * N, 1)
     const int g0 = (int)((long long)blockIdx.x * ngrid / gridDim.x);
     const int g1 = (int)((long long)(blockIdx.x + 1) * ngrid / gridDim.x);
     const float c = 0.5f * (float)(N - 1), ndl = -dx * 1.44269504088896340736f;
+    __shared__ float csn[kMaxViews];  // the share's grids (at most half the views)
+    for (int gi = g0 + tid; gi < g1; gi += NT) view_cos_sin(gi, V, &csn[2 * (gi - g0)], &csn[2 * (gi - g0) + 1]);
     for (int i = tid; i < 2 * IMG; i += NT) smem[i] = 0.0f;
     __syncthreads();
     load_image<N, NT, P>(img0, mu + (size_t)cand * N * N);
     __syncthreads();
     for (int gi = g0; gi < g1; ++gi) {
-        float cs, sn;
-        view_cos_sin(gi, V, &cs, &sn);
+        const float cs = csn[2 * (gi - g0)], sn = csn[2 * (gi - g0) + 1];
         for (int t = tid; t < (QUAD ? 4 : 2) * N; t += NT) {
             const int vi = t / N, j = t % N;
             yy[t] = dx * (y ? __ldg(y + ((size_t)cand * V + grid_view<QUAD>(gi, vi, V)) * N + grid_bin<N>(vi, j)) : 1.0f);

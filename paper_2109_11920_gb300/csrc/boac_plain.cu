@@ -49,12 +49,12 @@ __device__ __forceinline__ float ray_sample(const float* __restrict__ img, int n
 __global__ void attenuation_table_kernel(int n, int V, float dx, const float* __restrict__ mu,
                                          float* __restrict__ tab) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y, cand = blockIdx.z;
-    if (b >= n) return;
     const size_t nn = (size_t)n * n;
     const float* m_img = mu + cand * nn;
     float* t = tab + ((size_t)cand * V + v) * nn;
     float cs, sn;
-    view_cos_sin(v, V, &cs, &sn);
+    cta_view_cos_sin(v, V, &cs, &sn);
+    if (b >= n) return;
     const float c = 0.5f * (float)(n - 1);
     float suffix = 0.0f;
     walk_ray(
@@ -69,12 +69,12 @@ __global__ void attenuation_table_kernel(int n, int V, float dx, const float* __
 __global__ void project_otf_kernel(int n, int V, float dx, const float* __restrict__ mu,
                                    const float* __restrict__ F, float* __restrict__ q) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y, cand = blockIdx.z;
-    if (b >= n) return;
     const size_t nn = (size_t)n * n;
     const float* m_img = mu + cand * nn;
     const float* f_img = F + cand * nn;
     float cs, sn;
-    view_cos_sin(v, V, &cs, &sn);
+    cta_view_cos_sin(v, V, &cs, &sn);
+    if (b >= n) return;
     const float c = 0.5f * (float)(n - 1);
     float suffix = 0.0f, acc = 0.0f;
     walk_ray(
@@ -95,8 +95,7 @@ __global__ void project_otf_kernel(int n, int V, float dx, const float* __restri
 // where they fit: blockDim.y views of one candidate per CTA, a thread per ray.
 // Same operations and sums.  4 candidates of 100 x 100 and 75 views: a
 // projection from the table took 52 us through L1,
-// here 47; the whole 10 iterations 1.35 -> 1.30 ms, 18 projections of 128 x 128 and
-// 113 views with their back-projection 0.88 -> 0.82.
+// here 41.
 __device__ __forceinline__ const float* padded_image(float* smem, int slot, int n, const float* __restrict__ src) {
     const int P = n + 1, size = P * (n + 2) + 1;
     float* img = smem + slot * size;
@@ -104,8 +103,10 @@ __device__ __forceinline__ const float* padded_image(float* smem, int slot, int 
     for (int i = tid; i < P; i += nt) img[i] = img[(n + 1) * P + i] = 0.0f;
     for (int i = tid; i <= n + 1; i += nt) img[i * P] = 0.0f;
     if (tid == 0) img[size - 1] = 0.0f;
+    const int j = threadIdx.x;  // blockDim.x >= n
+#pragma unroll 8
     for (int r = threadIdx.y; r < n; r += blockDim.y)
-        for (int j = threadIdx.x; j < n; j += blockDim.x) img[(r + 1) * P + j + 1] = __ldg(src + (size_t)r * n + j);
+        if (j < n) img[(r + 1) * P + j + 1] = __ldg(src + (size_t)r * n + j);
     return img;
 }
 __device__ __forceinline__ float ray_sample_padded(const float* img, int n, int k, int b, float cs, float sn, float c) {
@@ -114,6 +115,7 @@ __device__ __forceinline__ float ray_sample_padded(const float* img, int n, int 
     return bilerp_padded(img, n + 1, n, u, w);
 }
 
+constexpr int kRayViews = 8;  // most views of a CTA
 enum class RayOp { kTable, kProjectTable, kProject };
 template <RayOp OP>
 __global__ void __launch_bounds__(1024) ray_smem_kernel(int n, int V, float dx, const float* __restrict__ mu,
@@ -127,10 +129,11 @@ __global__ void __launch_bounds__(1024) ray_smem_kernel(int n, int V, float dx, 
     int slots = 0;
     if (OP != RayOp::kProjectTable) m_img = padded_image(smem, slots++, n, mu + cand * nn);
     if (OP != RayOp::kTable) f_img = padded_image(smem, slots++, n, F + cand * nn);
+    __shared__ float csn[kRayViews][2];  // one float64 sine and cosine per view, not per thread
+    if (b == 0) view_cos_sin(v, V, &csn[threadIdx.y][0], &csn[threadIdx.y][1]);
     __syncthreads();
     if (b >= n || v >= V) return;
-    float cs, sn;
-    view_cos_sin(v, V, &cs, &sn);
+    const float cs = csn[threadIdx.y][0], sn = csn[threadIdx.y][1];
     const float c = 0.5f * (float)(n - 1);
     const size_t plane = ((size_t)cand * V + v) * nn;
     float suffix = 0.0f, acc = 0.0f;
@@ -192,7 +195,7 @@ static bool ray_smem_launch(int n, int V, int B, float dx, const float* mu, cons
     int views = (int)((long long)V * B / sms);  // about one CTA per SM ...
     if (views < 2) views = 2;
     if (views > 1024 / width) views = 1024 / width;  // ... of at most 1024 threads
-    if (views > 8) views = 8;
+    if (views > kRayViews) views = kRayViews;
     if (views < 1) views = 1;
     if (views > V) views = V;
     ray_smem_kernel<OP><<<dim3((V + views - 1) / views, B), dim3(width, views), smem, st>>>(n, V, dx, mu, F, tab, out);
@@ -217,12 +220,12 @@ void project_table_rays(const boac_geom* g, int B, float dx, const float* tab, c
 __global__ void project_table_kernel(int n, int V, float dx, const float* __restrict__ tab,
                                      const float* __restrict__ F, float* __restrict__ q) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y, cand = blockIdx.z;
-    if (b >= n) return;
     const size_t nn = (size_t)n * n;
     const float* t = tab + ((size_t)cand * V + v) * nn;
     const float* f_img = F + cand * nn;
     float cs, sn;
-    view_cos_sin(v, V, &cs, &sn);
+    cta_view_cos_sin(v, V, &cs, &sn);
+    if (b >= n) return;
     const float c = 0.5f * (float)(n - 1);
     float acc = 0.0f;
     walk_ray(
@@ -238,7 +241,7 @@ __global__ void project_table_kernel(int n, int V, float dx, const float* __rest
 // out once for C candidates; kViewLanes lanes of a warp take a pixel's views
 // in turn, and every one of them adds up all views' sums in view order (one
 // thread per pixel left the GPU waiting: 4 candidates of 100 x 100 and 75
-// views: 196 -> 72 us).
+// views: 196 -> 67 us).
 constexpr int kViewLanes = 8;
 template <int C>
 __global__ void __launch_bounds__(kPixThreads)
@@ -282,22 +285,30 @@ __global__ void __launch_bounds__(kPixThreads)
                 float bacc[C];
 #pragma unroll
                 for (int q = 0; q < C; ++q) bacc[q] = 0.0f;
+                // the weights of the three samples, their loads in flight
+                // together, then the sums
+                float wt[3], t[3][C];
 #pragma unroll
                 for (int dk = 0; dk < 3; ++dk) {
                     const int k = kmin + dk;
-                    float wt = 0.0f;
+                    wt[dk] = 0.0f;
                     if (k <= kmax) {
                         float u, w;
                         sample_uw(k, b, cs, sn, c, &u, &w);
-                        wt = pixel_weight(u, w, i, j, n);
-                    }
-                    if (wt != 0.0f) {
-                        const float* t = tab + ((size_t)cand0 * V + v) * nn + (size_t)k * n + b;
-#pragma unroll
-                        for (int q = 0; q < C; ++q)
-                            if (C == 1 || cand0 + q < B) bacc[q] = fmaf(wt, __ldg(t + (size_t)q * V * nn), bacc[q]);
+                        wt[dk] = pixel_weight(u, w, i, j, n);
                     }
                 }
+                const float* tp = tab + ((size_t)cand0 * V + v) * nn + (size_t)kmin * n + b;
+#pragma unroll
+                for (int dk = 0; dk < 3; ++dk)
+#pragma unroll
+                    for (int q = 0; q < C; ++q)
+                        t[dk][q] = wt[dk] != 0.0f && (C == 1 || cand0 + q < B) ? __ldg(tp + (size_t)q * V * nn + dk * n) : 0.0f;
+#pragma unroll
+                for (int dk = 0; dk < 3; ++dk)
+                    if (wt[dk] != 0.0f)
+#pragma unroll
+                        for (int q = 0; q < C; ++q) bacc[q] = fmaf(wt[dk], t[dk][q], bacc[q]);
 #pragma unroll
                 for (int q = 0; q < C; ++q)
                     if (C == 1 || cand0 + q < B)

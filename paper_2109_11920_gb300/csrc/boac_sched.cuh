@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(256) scatter_schedule_kernel(int V, unsigned s
     __shared__ int num[1024], start[1024], cur[1024];
     __shared__ int s_rounds;
     float cs, sn;
-    view_cos_sin(gi, V, &cs, &sn);  // grid gi's base view, as in the fused kernel
+    cta_view_cos_sin(gi, V, &cs, &sn);  // grid gi's base view, as in the fused kernel
     const float c = 0.5f * (float)(N - 1);
     unsigned short* out = sched + ((size_t)gi * 9 + cls) * S::CLS_ENTRIES;
     for (int i = threadIdx.x; i < 1024; i += blockDim.x) num[i] = 0;

@@ -109,7 +109,7 @@ __device__ void block_sort(int* key, int* val, int P) {
 __device__ int row_pairs(int n, int V, int row, int* key, int P, int* sh32) {
     const int v = row / n, b = row % n;
     float cs, sn;
-    view_cos_sin(v, V, &cs, &sn);
+    cta_view_cos_sin(v, V, &cs, &sn);
     const float c = 0.5f * (float)(n - 1);
     int valid = 0;
     for (int t = threadIdx.x; t < P; t += blockDim.x) {
