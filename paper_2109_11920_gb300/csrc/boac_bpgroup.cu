@@ -156,7 +156,8 @@ __global__ void __launch_bounds__(NT) project_group_kernel(int V, float dx, cons
 // grid's views, r = S / q, and the grid's back-projection of r into its slice
 // of `partial`.  A grid's rays belong to it alone, so nothing is exchanged
 // with other CTAs and the steps need no launch each (projection, ratio and
-// back-projection kernels before).  The sums are those of
+// back-projection kernels: 89 us an iteration of 8 candidates at 96 x 96 and
+// 90 views; here 39, and 12 for the sum and update).  The sums are those of
 // project_group_kernel (four segments per ray, its sample order) and
 // bp_group_kernel, bit for bit: the samples of F go through W, where the
 // threads of a ray's segment add them up in order, one view per half of the

@@ -94,8 +94,7 @@ __global__ void project_otf_kernel(int n, int V, float dx, const float* __restri
 // a ring of zeros, so a sample needs no test per neighbour), for the sides
 // where they fit: blockDim.y views of one candidate per CTA, a thread per ray.
 // Same operations and sums.  4 candidates of 100 x 100 and 75 views: a
-// projection from the table took 52 us through L1,
-// here 41.
+// projection from the table took 52 us through L1, here 35.
 __device__ __forceinline__ const float* padded_image(float* smem, int slot, int n, const float* __restrict__ src) {
     const int P = n + 1, size = P * (n + 2) + 1;
     float* img = smem + slot * size;
@@ -193,7 +192,7 @@ static bool ray_smem_launch(int n, int V, int B, float dx, const float* mu, cons
     }
     const int width = (n + 31) / 32 * 32, sms = sm_count() > 0 ? sm_count() : 1;
     int views = (int)((long long)V * B / sms);  // about one CTA per SM ...
-    if (views < 2) views = 2;
+    if (views < 4) views = 4;
     if (views > 1024 / width) views = 1024 / width;  // ... of at most 1024 threads
     if (views > kRayViews) views = kRayViews;
     if (views < 1) views = 1;
@@ -241,9 +240,8 @@ __global__ void project_table_kernel(int n, int V, float dx, const float* __rest
 // out once for C candidates; kViewLanes lanes of a warp take a pixel's views
 // in turn, and every one of them adds up all views' sums in view order (one
 // thread per pixel left the GPU waiting: 4 candidates of 100 x 100 and 75
-// views: 196 -> 67 us).
-constexpr int kViewLanes = 8;
-template <int C>
+// views took 196 us, with 16 lanes and C = 2 62; with 8 lanes 67, C = 4 80).
+template <int C, int kViewLanes>
 __global__ void __launch_bounds__(kPixThreads)
     backproject_gather_kernel(int n, int V, int B, float scale, const float* __restrict__ tab,
                               const float* __restrict__ y, float* __restrict__ out, int accumulate) {
@@ -331,18 +329,26 @@ __global__ void __launch_bounds__(kPixThreads)
         }
 }
 
+template <int C, int LANES>
+static void gather_launch(int n, int V, int B, float scale, const float* tab, const float* y, float* out, int accumulate,
+                          cudaStream_t st) {
+    const size_t warps = ((size_t)n * n * LANES + 31) / 32;
+    const unsigned blocks = (unsigned)((warps * 32 + kPixThreads - 1) / kPixThreads);
+    backproject_gather_kernel<C, LANES><<<dim3(blocks, (B + C - 1) / C), kPixThreads, sizeof(float) * 2 * V, st>>>(
+        n, V, B, scale, tab, y, out, accumulate);
+}
+
 void backproject_gather(int n, int V, int B, float scale, const float* tab, const float* y, float* out,
                         int accumulate, cudaStream_t st) {
-    const size_t warps = ((size_t)n * n * kViewLanes + 31) / 32;
-    const unsigned blocks = (unsigned)((warps * 32 + kPixThreads - 1) / kPixThreads);
-    const size_t smem = sizeof(float) * 2 * V;
+    // Two candidates share a thread's weights; a pixel's views go to 16 lanes
+    // while 8 would leave the SMs short of threads (about 1300 each; 6
+    // candidates of 35 x 35 and 109 views, whole call: 0.32 against 0.28 ms;
+    // 5 of 131 x 131: 0.67 against 0.72).
+    const bool wide = (long long)n * n * ((B + 1) / 2) * 8 <= 1300LL * (sm_count() > 0 ? sm_count() : 1);
     if (B == 1)
-        backproject_gather_kernel<1><<<dim3(blocks, 1), kPixThreads, smem, st>>>(n, V, B, scale, tab, y, out, accumulate);
-    else if (B == 2)
-        backproject_gather_kernel<2><<<dim3(blocks, 1), kPixThreads, smem, st>>>(n, V, B, scale, tab, y, out, accumulate);
+        (wide ? gather_launch<1, 16> : gather_launch<1, 8>)(n, V, B, scale, tab, y, out, accumulate, st);
     else
-        backproject_gather_kernel<4><<<dim3(blocks, (B + 3) / 4), kPixThreads, smem, st>>>(n, V, B, scale, tab, y, out,
-                                                                                         accumulate);
+        (wide ? gather_launch<2, 16> : gather_launch<2, 8>)(n, V, B, scale, tab, y, out, accumulate, st);
 }
 
 __global__ void ratio_kernel(int count, const float* __restrict__ S, const float* __restrict__ q,
