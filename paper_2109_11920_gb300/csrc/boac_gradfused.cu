@@ -295,16 +295,20 @@ __global__ void __launch_bounds__(8 * N, 1) grad_fused_kernel(GradFusedArgs a) {
             const float w13 = dx * k1[2 * N + k], w14 = dx * k1[3 * N + k];
             const float w23 = Y ? dx * k2[2 * N + k] : 0.0f, w24 = Y ? dx * k2[3 * N + k] : 0.0f;
             float q3 = 0.0f, p4 = 0.0f;
-#pragma unroll 1
+#pragma unroll 2
             for (int s4 = 0; s4 < SEG; s4 += 4) {
-                float e[8];
+                // the stored samples of four steps in flight together (64
+                // candidates x 10 iterations: 8.08 -> 7.99 ms)
+                float yy[4], e[8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) yy[j] = Y ? __ldcg(Yc + (k0 + s4 + j) * N + k) : 0.0f;
                 tmem_ld8(stash + 2 * (SEG + s4), e);
                 tmem_wait_ld(e);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int b = k0 + s4 + j;
                     const float x = W[k * WP + b];
-                    const float yv = Y ? __ldcg(Yc + b * N + k) : 0.0f;
+                    const float yv = yy[j];
                     const float a3 = e[2 * j] * fmaf(w23, yv, w13 * x);
                     const float a4 = e[2 * j + 1] * fmaf(w24, yv, w14 * x);
                     q3 += a3;
