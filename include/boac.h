@@ -192,21 +192,23 @@ int boac_rasterize_mu_params(const boac_geom *g, const float *p, int B,
 /* ---- Eq. 1-2: forward projection q = A^mu F ----------------------------
  *   mu  [B][n][n], F [B][n][n]   (device, float32)
  *   q   [B][n_views][n_bins]     output (device, float32)
- * The attenuation is integrated along each ray on the fly; no workspace. */
+ * The attenuation is integrated along each ray on the fly (for n = 64, 96, 128
+ * with an even view count once for the views that share a sample grid); no
+ * workspace. */
 int boac_project(const boac_geom *g, const float *mu, const float *F, int B,
                  float *q, void *stream);
 
 /* ---- Eq. 2 adjoint: out = (A^mu)^T y -----------------------------------
  * Exact transpose of boac_project (same bilinear weights), deterministic:
  * for n = 64, 96, 128 with an even view count a race-free scatter of the
- * views that share a sample grid into per-grid images summed in grid order,
- * for other sizes a per-pixel gather.
+ * views that share a sample grid into partial images (one per CTA's run of
+ * grids) summed in order, for other sizes a per-pixel gather.
  *   y   [B][n_views][n_bins] (device, float32); NULL means y = 1 everywhere
  *       (the MLEM sensitivity image)
  *   out [B][n][n]            output (device, float32)
  *   ws  workspace of boac_workspace_bytes(g, B, BOAC_OP_BACKPROJECT) bytes
- *       (holds the attenuation factors of every ray sample and the per-grid
- *       images). */
+ *       (holds partial images and, for sizes without the scatter, the
+ *       attenuation factors of every ray sample). */
 int boac_backproject(const boac_geom *g, const float *mu, const float *y,
                      int B, float *out, void *ws, size_t ws_bytes,
                      void *stream);
@@ -241,10 +243,12 @@ int boac_backproject(const boac_geom *g, const float *mu, const float *y,
 int boac_mlem(const boac_geom *g, const float *mu, const float *S,
               long long s_stride, float *F, int K, int B, double *L,
               int include_lgamma, void *ws, size_t ws_bytes, void *stream);
-/* boac_mlem_unfused: the same MLEM over the whole batch with one launch per
- * step (attenuation table once; per iteration the grouped projector, the
- * ratio, the grouped back-projection and the update, each covering every
- * candidate, so one candidate spreads over many CTAs).  Same arguments,
+/* boac_mlem_unfused: the same MLEM over the whole batch from attenuation
+ * tables written once, a few launches per iteration that each cover every
+ * candidate, so one candidate spreads over many CTAs (n = 64, 96, 128 with an
+ * even view count: one kernel for a sample grid's projection, ratio and
+ * back-projection, one for the sum over grids and the update; else one per
+ * step).  Same arguments,
  * conventions and errors as boac_mlem, except that any view count is
  * accepted (boac_mlem needs an even one); workspace boac_workspace_bytes(g,
  * B, BOAC_OP_MLEM_UNFUSED) (the attenuation tables, 4 n_views n^2 bytes per
@@ -267,7 +271,9 @@ int boac_mlem_plain(const boac_geom *g, const float *mu, const float *S,
  * F [n][n] (in: initial image, out: F^K) in three caller-owned device pools.
  * Its score (Eq. 5, as boac_mlem) goes to L[index in cands].  Per class, one
  * persistent fused kernel takes candidates from a work queue, largest K
- * first.  config[c] (host array, or NULL for defaults) picks class c's launch
+ * first; the classes' kernels run at once and share the SMs (programmatic
+ * dependent launches in `stream`, which work enqueued after the call waits
+ * for as usual).  config[c] (host array, or NULL for defaults) picks class c's launch
  * shape: 2 * shape + pair, shape 0/1/2 = CTAs of 2n/4n/8n (<= 1024) threads,
  * pair = 1 for two views per sample grid instead of four (four needs
  * n_views % 4 == 0); with n_views % 4 == 0, configurations 6, 7 and 8 run

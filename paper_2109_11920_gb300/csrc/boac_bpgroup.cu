@@ -1,6 +1,6 @@
 // boac_bpgroup.cu -- grouped projection and back-projection (Eq. 2 and its
-// adjoint) for the unfused paths -- boac_backproject, the launch-per-step
-// MLEM and the gradient -- from a table of attenuation factors
+// adjoint) for the unfused paths -- the launch-per-step MLEM, the batched
+// unfused MLEM and the batched gradient -- from a table of attenuation factors
 // tab[cand][v][k][b]:
 //
 //   q[cand][v][b] = dx * sum_k tab_v[k][b] F(sample (k, b) of view v)

@@ -6,10 +6,14 @@
 // One CTA owns one candidate at a time and keeps its whole state on chip:
 //   img0  F (padded n+2 rows x n+1 floats, zero ring)   -- mu during set-up
 //   img1  back-projection accumulator (same layout)
-//   W     n x (n+1) ray-sample buffer (F samples, then G = dx a r)
+//   W     n x (n+4) ray-sample buffer (F samples, then G = dx a r)
+// and in its SM's tensor memory the attenuation of the grid in flight.
 // The candidate's "system matrix" -- the attenuation of every ray sample --
 // is built once per candidate into a per-CTA slot of the workspace (as
-// exp2 exponents) and read back, coalesced, in every iteration.
+// exp2 exponents) and read back, coalesced, in every iteration: the next
+// grid's exponents go into tensor memory while this grid is scattered, and
+// the factors taken from them in the forward passes stay there for the
+// back-projection weights.
 //
 // Four views share one sample grid: with bins and ray samples on the pixel
 // pitch, the grids of phi, phi + pi/2, phi + pi and phi + 3pi/2 are the same

@@ -4,7 +4,8 @@
 //
 // Ray kernels run one thread per (candidate, view, bin) and walk the ray from
 // the detector side (k = n-1) inwards, so the attenuation suffix sum of
-// Eq. 1's inner integral is a running register sum.  The back-projector is a
+// Eq. 1's inner integral is a running register sum; the images are in shared
+// memory where they fit (ray_smem_kernel).  The back-projector is a
 // per-pixel gather over the <= 3 x 3 ray samples whose bilinear footprint
 // contains the pixel, with the weights recomputed exactly as the projector
 // computes them (sample_uw + pixel_weight), so no atomics are needed and the

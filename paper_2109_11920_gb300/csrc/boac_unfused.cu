@@ -1,6 +1,9 @@
-// boac_unfused.cu -- MLEM for a batch of candidates with one launch per step
-// of the iteration (attenuation table once; per iteration q = A F, r = S / q,
-// z = A^T r, F <- F z / sens), every launch covering the whole batch.  Where
+// boac_unfused.cu -- MLEM for a batch of candidates from a table of attenuation
+// factors (written once), every launch covering the whole batch: per iteration
+// two launches for 64 / 96 / 128 images with an even view count (q, r and the
+// back-projection of every sample grid, then the sum over grids and the
+// update), else one launch per step (q = A F, r = S / q, z = A^T r,
+// F <- F z / sens).  Where
 // the batch is too small to fill the GPU with the fused kernel's one CTA (or
 // one cluster) per candidate, these kernels spread one candidate over many
 // CTAs (one per sample grid in the projector and the back-projector) and
