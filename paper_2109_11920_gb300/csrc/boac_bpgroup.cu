@@ -161,14 +161,16 @@ __global__ void __launch_bounds__(NT) project_group_kernel(int V, float dx, cons
 // project_group_kernel (four segments per ray, its sample order) and
 // bp_group_kernel, bit for bit: the samples of F go through W, where the
 // threads of a ray's segment add them up in order, one view per half of the
-// CTA; the scatter runs in schedule order.
+// CTA; the scatter runs in schedule order where a schedule is kept (SCHED),
+// in lattice order elsewhere (the same sums: building one for each call costs
+// more than its few scatters gain).
 template <int N, bool QUAD>
 struct GroupStep {
     static constexpr int NT = 8 * N, P = N + 1, WP = N + 1;
     static constexpr int IMG = (N + 1) * (N + 2) + 1 + kScatterPad;
     static constexpr size_t SMEM = sizeof(float) * ((size_t)IMG + (size_t)N * WP + 16 * N + 4 * N);
 };
-template <int N, bool QUAD>
+template <int N, bool QUAD, bool SCHED>
 __global__ void __launch_bounds__(8 * N, N <= 96 ? 2 : 1)
     mlem_group_kernel(int V, float dx, const float* __restrict__ tab, const float* __restrict__ S, long long s_stride,
                       const float* __restrict__ F, const unsigned short* __restrict__ sched,
@@ -188,7 +190,7 @@ __global__ void __launch_bounds__(8 * N, N <= 96 ? 2 : 1)
     const float* tb = tab + (size_t)cand * V * nn;
     const float* f = F + (size_t)cand * nn;
     const float* Sc = S + (size_t)cand * s_stride;
-    const unsigned short* gs = sched + (size_t)gi * 9 * SchedShape<N>::CLS_ENTRIES;
+    const unsigned short* gs = SCHED ? sched + (size_t)gi * 9 * SchedShape<N>::CLS_ENTRIES : nullptr;
     for (int i = tid; i < IMG; i += NT) img[i] = 0.0f;
     __syncthreads();
 #pragma unroll 4
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(8 * N, N <= 96 ? 2 : 1)
     }
     __syncthreads();
     SchedSlots<N, NT> sched0;
-    sched0.load(gs);
+    if constexpr (SCHED) sched0.load(gs);
     {
         const float y1 = rr[lb], y2 = rr[N + (N - 1 - lb)];
 #pragma unroll 4
@@ -260,7 +262,8 @@ __global__ void __launch_bounds__(8 * N, N <= 96 ? 2 : 1)
         }
     }
     __syncthreads();
-    scatter_scheduled<N, NT, P, WP, true>(W, img, cs, sn, c, gs, sched0);
+    if constexpr (SCHED) scatter_scheduled<N, NT, P, WP, true>(W, img, cs, sn, c, gs, sched0);
+    else scatter_classes<N, NT, P, WP>(W, img, cs, sn, c);
     float* out = partial + ((size_t)cand * ngrid + gi) * nn;
     for (int i = tid; i < (int)nn; i += NT) out[i] = img[(i / N + 1) * P + (i % N) + 1];
 }
@@ -385,7 +388,7 @@ int project_table(const boac_geom* g, int B, const float* tab, const float* F, f
     return s;
 }
 
-template <int N, bool QUAD>
+template <int N, bool QUAD, bool SCHED>
 static int mlem_group_launch(int V, int B, float dx, const float* tab, const float* S, long long s_stride,
                              const float* F, const unsigned short* sched, float* partial, cudaStream_t st) {
     constexpr size_t smem = GroupStep<N, QUAD>::SMEM;
@@ -394,13 +397,13 @@ static int mlem_group_launch(int V, int B, float dx, const float* tab, const flo
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDev) return launch_status();
     if (!attr_set[dev]) {
-        if (cudaFuncSetAttribute(mlem_group_kernel<N, QUAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(mlem_group_kernel<N, QUAD, SCHED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem) != cudaSuccess)
             return launch_status();
         attr_set[dev] = true;
     }
-    mlem_group_kernel<N, QUAD><<<dim3(QUAD ? V / 4 : V / 2, B), 8 * N, smem, st>>>(V, dx, tab, S, s_stride, F, sched,
-                                                                                 partial);
+    mlem_group_kernel<N, QUAD, SCHED>
+        <<<dim3(QUAD ? V / 4 : V / 2, B), 8 * N, smem, st>>>(V, dx, tab, S, s_stride, F, sched, partial);
     return launch_status();
 }
 
@@ -411,13 +414,9 @@ int sum_partial_images(int B, int shares, int nn, const float* partial, float* o
 
 bool mlem_grouped(const boac_geom* g) { return bp_grouped(g); }
 
-size_t mlem_group_sched_bytes(const boac_geom* g) {
-    return bp_grouped(g) ? sched_bytes(g->n, g->n_views % 4 == 0 ? g->n_views / 4 : g->n_views / 2) : 0;
-}
-
-const unsigned short* mlem_group_sched(const boac_geom* g, unsigned short* ws, cudaStream_t st, int* status) {
+const unsigned short* mlem_group_sched(const boac_geom* g, cudaStream_t st, int* status) {
     const int V = g->n_views;
-    return sched_prepare(g->n, V, V % 4 == 0 ? V / 4 : V / 2, g->n + 1 /* GroupStep<N>::WP */, ws, st, status);
+    return sched_prepare(g->n, V, V % 4 == 0 ? V / 4 : V / 2, g->n + 1 /* GroupStep<N>::WP */, nullptr, st, status);
 }
 
 int mlem_group_iteration(const boac_geom* g, int B, float dx, const float* tab, const float* S, long long s_stride,
@@ -425,10 +424,12 @@ int mlem_group_iteration(const boac_geom* g, int B, float dx, const float* tab, 
     const int n = g->n, V = g->n_views;
     const bool quad = V % 4 == 0;
     int s = BOAC_EUNSUPPORTED;
-#define X(NV)                                                                                      \
-    if (n == NV)                                                                                   \
-        s = quad ? mlem_group_launch<NV, true>(V, B, dx, tab, S, s_stride, F, sched, partial, st)  \
-                 : mlem_group_launch<NV, false>(V, B, dx, tab, S, s_stride, F, sched, partial, st);
+#define X(NV)                                                                                               \
+    if (n == NV) {                                                                                          \
+        auto launch = sched ? (quad ? mlem_group_launch<NV, true, true> : mlem_group_launch<NV, false, true>)   \
+                            : (quad ? mlem_group_launch<NV, true, false> : mlem_group_launch<NV, false, false>); \
+        s = launch(V, B, dx, tab, S, s_stride, F, sched, partial, st);                                      \
+    }
     X(64) X(96) X(128)
 #undef X
     if (s != BOAC_OK) return s;

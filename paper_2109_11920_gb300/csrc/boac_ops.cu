@@ -182,8 +182,13 @@ __global__ void __launch_bounds__(8 * N, 1)
     }
 }
 
-// z of grids [blockIdx.x share) of candidate blockIdx.y into its partial image.
-template <int N, bool QUAD>
+// z of grids [blockIdx.x share) of candidate blockIdx.y into its partial
+// image.  SCHED: the scatter runs in the order of a kept schedule; elsewhere
+// in lattice order, with the same sums (one image at 128 x 128 and 120 views: a
+// schedule of the call's own takes about 190 us to build, all else 33 us;
+// 8 images with 230 views in lattice order, both operators: 297 us, with the
+// per-ray and per-grid table kernels 630).
+template <int N, bool QUAD, bool SCHED>
 __global__ void __launch_bounds__(8 * N, 1)
     backproject_grids_kernel(int V, float dx, const float* __restrict__ mu, const float* __restrict__ y,
                              const unsigned short* __restrict__ sched, float* __restrict__ partial) {
@@ -249,9 +254,9 @@ __global__ void __launch_bounds__(8 * N, 1)
         }
 #pragma unroll
         for (int s = 0; s < SEG; ++s) W[(k0 + s) * WP + lb] = gc[s];
-        const unsigned short* gs = sched + (size_t)gi * 9 * SchedShape<N>::CLS_ENTRIES;
+        const unsigned short* gs = SCHED ? sched + (size_t)gi * 9 * SchedShape<N>::CLS_ENTRIES : nullptr;
         SchedSlots<N, NT> sched0;
-        sched0.load(gs);
+        if constexpr (SCHED) sched0.load(gs);
         __syncthreads();
         if (QUAD) {
             const float y3 = yy[2 * N + lb], y4 = yy[3 * N + lb];
@@ -267,7 +272,8 @@ __global__ void __launch_bounds__(8 * N, 1)
             }
             __syncthreads();
         }
-        scatter_scheduled<N, NT, P, WP>(W, img1, cs, sn, c, gs, sched0);
+        if constexpr (SCHED) scatter_scheduled<N, NT, P, WP>(W, img1, cs, sn, c, gs, sched0);
+        else scatter_classes<N, NT, P, WP>(W, img1, cs, sn, c);
     }
     float* out = partial + ((size_t)cand * gridDim.x + blockIdx.x) * N * N;
     for (int i = tid; i < N * N; i += NT) out[i] = img1[(i / N + 1) * P + (i % N) + 1];
@@ -315,15 +321,16 @@ int project_t(int V, float dx, const float* mu, const float* F, int B, float* q,
 
 template <int N, bool QUAD>
 int backproject_t(int V, float dx, const float* mu, const float* y, int B, float* out, float* partial,
-                  unsigned short* sched_ws, cudaStream_t st) {
-    static bool done[64];
-    int s = allow_smem(backproject_grids_kernel<N, QUAD>, OpShape<N>::SMEM, done);
-    if (s != BOAC_OK) return s;
+                  cudaStream_t st) {
+    static bool done[2][64];
+    int s = BOAC_OK;
     const int ngrid = QUAD ? V / 4 : V / 2, shares = grid_shares(B, ngrid);
-    const unsigned short* sched = sched_prepare(N, V, ngrid, OpShape<N>::WP, sched_ws, st, &s);
+    const unsigned short* sched = sched_prepare(N, V, ngrid, OpShape<N>::WP, nullptr, st, &s);
     if (s != BOAC_OK) return s;
-    backproject_grids_kernel<N, QUAD>
-        <<<dim3(shares, B), 8 * N, OpShape<N>::SMEM, st>>>(V, dx, mu, y, sched, partial);
+    auto kernel = sched ? backproject_grids_kernel<N, QUAD, true> : backproject_grids_kernel<N, QUAD, false>;
+    s = allow_smem(kernel, OpShape<N>::SMEM, done[sched != nullptr]);
+    if (s != BOAC_OK) return s;
+    kernel<<<dim3(shares, B), 8 * N, OpShape<N>::SMEM, st>>>(V, dx, mu, y, sched, partial);
     return sum_partial_images(B, shares, N * N, partial, out, st);
 }
 
@@ -349,9 +356,9 @@ int project_on_grids(const boac_geom* g, const float* mu, const float* F, int B,
 }
 
 int backproject_on_grids(const boac_geom* g, const float* mu, const float* y, int B, float* out, float* partial,
-                         unsigned short* sched_ws, cudaStream_t st) {
+                         cudaStream_t st) {
     const bool quad = g->n_views % 4 == 0;
-#define CALL(NV, QUAD) backproject_t<NV, QUAD>(g->n_views, g->pixel_cm, mu, y, B, out, partial, sched_ws, st)
+#define CALL(NV, QUAD) backproject_t<NV, QUAD>(g->n_views, g->pixel_cm, mu, y, B, out, partial, st)
     BOAC_OPS(CALL)
 #undef CALL
 }

@@ -10,9 +10,9 @@ namespace boac {
 // Whether the geometry has these kernels (64 / 96 / 128 images, even views).
 bool ops_on_grids(const boac_geom* g);
 int project_on_grids(const boac_geom* g, const float* mu, const float* F, int B, float* q, cudaStream_t st);
-// partial: bp_partial_floats(g, B) floats; sched_ws: sched_bytes of scratch.
+// partial: bp_partial_floats(g, B) floats.
 int backproject_on_grids(const boac_geom* g, const float* mu, const float* y, int B, float* out, float* partial,
-                         unsigned short* sched_ws, cudaStream_t st);
+                         cudaStream_t st);
 // out[cand] = sum over shares of partial[cand][share], in order (boac_bpgroup.cu).
 int sum_partial_images(int B, int shares, int nn, const float* partial, float* out, cudaStream_t st);
 

@@ -540,9 +540,9 @@ extern "C" int boac_backproject(const boac_geom* g, const float* mu, const float
         base + align256(sizeof(float) * (size_t)chunk * g->n_views * nn));
     for (int c0 = 0; c0 < B; c0 += chunk) {
         const int cb = (B - c0) < chunk ? (B - c0) : chunk;
-        if (ops_on_grids(g)) {  // no table: its room holds the schedule if the cache has none
+        if (ops_on_grids(g)) {  // no table
             const int s = backproject_on_grids(g, mu + c0 * nn, y ? y + (size_t)c0 * g->n_views * g->n_bins : nullptr, cb,
-                                               out + c0 * nn, partial, reinterpret_cast<unsigned short*>(base), st);
+                                               out + c0 * nn, partial, st);
             if (s != BOAC_OK) return s;
             continue;
         }

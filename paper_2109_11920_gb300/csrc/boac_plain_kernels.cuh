@@ -62,10 +62,9 @@ int project_table(const boac_geom* g, int B, const float* tab, const float* F, f
                   cudaStream_t st);
 // One whole MLEM iteration F <- F A^T(S / A F) / sens from the table, for
 // geometries with grouped kernels (mlem_grouped): two launches, `partial` as
-// above, sched from mlem_group_sched (ws: mlem_group_sched_bytes of scratch).
+// above, sched from mlem_group_sched (nullptr where none is kept).
 bool mlem_grouped(const boac_geom* g);
-size_t mlem_group_sched_bytes(const boac_geom* g);
-const unsigned short* mlem_group_sched(const boac_geom* g, unsigned short* ws, cudaStream_t st, int* status);
+const unsigned short* mlem_group_sched(const boac_geom* g, cudaStream_t st, int* status);
 int mlem_group_iteration(const boac_geom* g, int B, float dx, const float* tab, const float* S, long long s_stride,
                          float* F, const float* sens, const unsigned short* sched, float* partial, cudaStream_t st);
 int backproject_table(const boac_geom* g, int B, const float* tab, const float* y, float scale, float* out,

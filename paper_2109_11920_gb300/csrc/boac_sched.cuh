@@ -219,11 +219,11 @@ inline int sched_launch(int n, int V, int ngrid, int wp, unsigned short* sched, 
 }
 
 // The schedule of geometry (n, V, ngrid) and sample-buffer pitch wp for a
-// launch on stream st: a slot of the device-side cache (built there when its
-// tag does not name the geometry and pitch), or, when no slot is free or the
-// schedule is larger than a slot, built into ws (sched_bytes(n, ngrid) bytes
-// of the caller's workspace).  Returns the schedule's address; *status is
-// BOAC_OK or the launch error.
+// launch on stream st: a kept one (built there when its tag does not name the
+// geometry and pitch), or, when there is no room for it, built into ws
+// (sched_bytes(n, ngrid) bytes of the caller's workspace).  Returns the
+// schedule's address, or nullptr where none is kept and ws is nullptr;
+// *status is BOAC_OK or the launch error.
 const unsigned short* sched_prepare(int n, int V, int ngrid, int wp, unsigned short* ws, cudaStream_t st,
                                     int* status);
 

@@ -3,20 +3,26 @@
 //
 // A schedule (boac_sched.cuh) depends on the image size, the view count,
 // the number of sample grids and the pitch of the kernel's sample buffer
-// only; building one takes about 0.27 ms at
-// 128 x 128 / 120 views, a tenth of a 16-candidate call.  The library keeps
-// kSchedCacheSlots schedules in static device memory, each slot with a
-// device-side tag naming the geometry it holds.  Static device memory is
-// zero when the module is loaded, so after a device reset every tag is
-// empty again and the next call rebuilds.  The host gives a geometry a slot
-// the first time it meets it on a device and never reassigns the slot, so
-// no call can read a schedule that another call is replacing.  Every call
-// launches the builder on its slot, whose CTAs return at once when the tag
-// already names the geometry, then a one-thread kernel that writes the tag
-// (after the build, in stream order).  Two calls on different streams that
-// both find the tag empty build the slot at the same time and write the
-// same values.  A geometry that finds no free slot, or whose schedule is
-// larger than a slot, is built into the caller's workspace on every call.
+// only; building one takes about 0.2 ms at 128 x 128 / 120 views, a tenth of
+// a 16-candidate call and more than the operators take.  The library keeps
+// schedules in an arena of static device memory, each with a device-side tag
+// naming the geometry it holds.  Static device memory is zero when the module
+// is loaded, so after a device reset every tag is empty again and the next
+// call rebuilds.  The host gives a geometry the next stretch of the arena, of
+// its schedule's size, the first time it meets it on a device and never
+// reassigns it, so no call can read a schedule that another call is
+// replacing.  Every call launches the builder on its stretch, whose CTAs
+// return at once when the tag already names the geometry, then a one-thread
+// kernel that writes the tag (after the build, in stream order).  Two calls
+// on different streams that both find the tag empty build the schedule at the
+// same time and write the same values.
+//
+// A geometry that finds no room, or whose schedule is larger than 4 MiB, has
+// no kept schedule: it is built into the caller's workspace on every call, or,
+// for the callers that give none because they scatter a few grids per call,
+// not at all.  (Eight fixed slots of 4 MiB held a program of nine geometries
+// no more: back-projections of one to eight 128 x 128 images then took 183 to
+// 305 us, most of it the build.)
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -28,12 +34,14 @@ namespace boac {
 
 namespace {
 
-constexpr int kSchedCacheSlots = 8;
-constexpr size_t kSchedCacheEntries = ((size_t)4 << 20) / sizeof(unsigned short);  // 4 MiB per slot
+constexpr int kSchedCacheSlots = 256;
+constexpr size_t kSchedArenaEntries = ((size_t)64 << 20) / sizeof(unsigned short);  // 58 of 1.1 MB (128 x 128, 120 views)
+constexpr size_t kSchedMaxBytes = (size_t)4 << 20;  // the largest schedule kept
 constexpr int kSchedCacheDevices = 64;
 
 struct SlotGeom {
     int n, V, ngrid, wp;  // n == 0: free
+    size_t at;            // its first entry in the arena
 };
 
 std::mutex g_sched_mu;
@@ -41,22 +49,29 @@ SlotGeom g_sched_geom[kSchedCacheDevices][kSchedCacheSlots];
 
 }  // namespace
 
-static __device__ __align__(256) unsigned short g_sched_cache[kSchedCacheSlots][kSchedCacheEntries];
+static __device__ __align__(256) unsigned short g_sched_cache[kSchedArenaEntries];
 static __device__ unsigned long long g_sched_tag[kSchedCacheSlots];
 
 __global__ void sched_tag_kernel(unsigned long long* tag, unsigned long long v) { *tag = v; }
 
-// The slot of (n, V, ngrid, wp) on device dev, assigning a free one; -1 if none.
-static int sched_slot_of(int dev, int n, int V, int ngrid, int wp) {
+// The slot of (n, V, ngrid, wp) on device dev, assigning the next one and the
+// arena's next entries (*at); -1 if either runs out.
+static int sched_slot_of(int dev, int n, int V, int ngrid, int wp, size_t* at) {
+    const size_t need = sched_bytes(n, ngrid) / sizeof(unsigned short);  // a multiple of 256 bytes
     std::lock_guard<std::mutex> lock(g_sched_mu);
+    size_t used = 0;
     // slots are filled in order and never freed, so no match follows a free slot
     for (int i = 0; i < kSchedCacheSlots; ++i) {
         SlotGeom& s = g_sched_geom[dev][i];
-        if (s.n == n && s.V == V && s.ngrid == ngrid && s.wp == wp) return i;
         if (s.n == 0) {
-            s = SlotGeom{n, V, ngrid, wp};
+            if (need > kSchedArenaEntries - used) return -1;
+            s = SlotGeom{n, V, ngrid, wp, used};
+        }
+        if (s.n == n && s.V == V && s.ngrid == ngrid && s.wp == wp) {
+            *at = s.at;
             return i;
         }
+        used = s.at + sched_bytes(s.n, s.ngrid) / sizeof(unsigned short);
     }
     return -1;
 }
@@ -64,21 +79,22 @@ static int sched_slot_of(int dev, int n, int V, int ngrid, int wp) {
 const unsigned short* sched_prepare(int n, int V, int ngrid, int wp, unsigned short* ws, cudaStream_t st,
                                     int* status) {
     int dev = -1, slot = -1;
-    if (sched_bytes(n, ngrid) <= sizeof(unsigned short) * kSchedCacheEntries && cudaGetDevice(&dev) == cudaSuccess &&
-        dev >= 0 && dev < kSchedCacheDevices)
-        slot = sched_slot_of(dev, n, V, ngrid, wp);
+    size_t at = 0;
+    if (sched_bytes(n, ngrid) <= kSchedMaxBytes && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 &&
+        dev < kSchedCacheDevices)
+        slot = sched_slot_of(dev, n, V, ngrid, wp, &at);
     void* base = nullptr;
     void* tags = nullptr;
     if (slot >= 0 && (cudaGetSymbolAddress(&base, g_sched_cache) != cudaSuccess ||
                       cudaGetSymbolAddress(&tags, g_sched_tag) != cudaSuccess || !base || !tags)) {
-        cudaGetLastError();  // not a sticky error: build into the workspace instead
+        cudaGetLastError();  // not a sticky error: as without a slot
         slot = -1;
     }
     if (slot < 0) {
-        *status = sched_launch(n, V, ngrid, wp, ws, st);
+        *status = ws ? sched_launch(n, V, ngrid, wp, ws, st) : BOAC_OK;
         return ws;
     }
-    unsigned short* sched = static_cast<unsigned short*>(base) + (size_t)slot * kSchedCacheEntries;
+    unsigned short* sched = static_cast<unsigned short*>(base) + at;
     unsigned long long* tag = static_cast<unsigned long long*>(tags) + slot;
     const unsigned long long want = sched_tag_value(n, V, ngrid, wp);
     *status = sched_launch(n, V, ngrid, wp, sched, st, tag, want);

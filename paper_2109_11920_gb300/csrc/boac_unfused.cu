@@ -19,7 +19,7 @@ namespace boac {
 namespace {
 
 struct UnfusedLayout {
-    size_t status, tab, sens, z, q, r, partial, sched, total;
+    size_t status, tab, sens, z, q, r, partial, total;
 };
 
 UnfusedLayout unfused_layout(const boac_geom* g, int B) {
@@ -38,7 +38,6 @@ UnfusedLayout unfused_layout(const boac_geom* g, int B) {
     l.q = take(Bs * vb);
     l.r = take(Bs * vb);
     l.partial = take(bp_partial_floats(g, B));
-    l.sched = take(mlem_group_sched_bytes(g) / sizeof(float));
     l.total = off;
     return l;
 }
@@ -67,13 +66,14 @@ int mlem_unfused(const boac_geom* g, const float* mu, const float* S, long long 
     int s = backproject_table(g, B, tab, nullptr, dx, sens, 0, partial, st);
     if (s != BOAC_OK) return s;
     const unsigned short* sched = nullptr;
-    if (K > 0 && mlem_grouped(g)) {
-        sched = mlem_group_sched(g, reinterpret_cast<unsigned short*>(base + l.sched), st, &s);
+    const bool grouped = mlem_grouped(g);
+    if (K > 0 && grouped) {
+        sched = mlem_group_sched(g, st, &s);
         if (s != BOAC_OK) return s;
     }
     for (int it = 0; it < K; ++it) {
         BOAC_RANGE("MLEM iteration");
-        if (sched) {
+        if (grouped) {
             s = mlem_group_iteration(g, B, dx, tab, S, s_stride, F, sens, sched, partial, st);
             if (s != BOAC_OK) return s;
             continue;
