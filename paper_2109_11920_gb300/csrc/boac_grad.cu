@@ -118,8 +118,8 @@ __global__ void __launch_bounds__(NT) abar_grid_kernel(int V, float dx, const fl
 
 // abar += dx (y1 (B X1) + y2 (B X2)) for B candidates: per grid for image
 // sides 64, 96, 128 and even view counts, else one thread per ray.
-static int abar_accum(const boac_geom* g, int B, float dx, const float* y1, const float* X1, const float* y2,
-                      const float* X2, float* abar, cudaStream_t st) {
+[[nodiscard]] static int abar_accum(const boac_geom* g, int B, float dx, const float* y1, const float* X1,
+                                    const float* y2, const float* X2, float* abar, cudaStream_t st) {
     const int n = g->n, V = g->n_views;
     if (!((n == 64 || n == 96 || n == 128) && V % 2 == 0)) {
         abar_accum_kernel<<<ray_grid(g, B), kRayThreads, 0, st>>>(n, V, dx, y1, X1, y2, X2, abar);
@@ -519,19 +519,23 @@ static int score_grad_run(const boac_geom* g, const boac_tissue* t, const float*
     const int g1p = grid_1d(cnt_pix, 256), g1b = grid_1d(cnt_bin, 256);
 
     // one MLEM step F_in -> F_out, leaving q, r and z = A^T r behind
-    auto mlem_step = [&](const float* F_in, float* F_o, float* q, float* r, float* z) {
-        project_table(g, B, tab, F_in, dx, q, st);
+    auto mlem_step = [&](const float* F_in, float* F_o, float* q, float* r, float* z) -> int {
+        int e = project_table(g, B, tab, F_in, dx, q, st);
+        if (e != BOAC_OK) return e;
         ratio_batched_kernel<<<g1b, 256, 0, st>>>(B, (int)vb, S, s_stride, q, r);
-        backproject_table(g, B, tab, r, dx, z, 0, partial, st);
+        e = backproject_table(g, B, tab, r, dx, z, 0, partial, st);
+        if (e != BOAC_OK) return e;
         cudaMemcpyAsync(F_o, F_in, sizeof(float) * cnt_pix, cudaMemcpyDeviceToDevice, st);
         update_kernel<<<g1p, 256, 0, st>>>((int)cnt_pix, F_o, z, sens);
+        return BOAC_OK;
     };
     // ---- forward
     NvtxPhases phase("gradient: forward MLEM with checkpoints");
     int s = rasterize_launch(g, t, c, t ? 6 : kParams, B, BOAC_RASTER_AREA, mu, st);
     if (s != BOAC_OK) return s;
     attenuation_table(g, B, mu, tab, st);
-    backproject_table(g, B, tab, nullptr, dx, sens, 0, partial, st);
+    s = backproject_table(g, B, tab, nullptr, dx, sens, 0, partial, st);
+    if (s != BOAC_OK) return s;
     cudaMemsetAsync(abar, 0, sizeof(float) * (size_t)B * V * nn, st);
     cudaMemsetAsync(sensbar, 0, sizeof(float) * cnt_pix, st);
     // F^0 = 1 into checkpoint 0; F^{j ckpt} into checkpoint j; F^K into Fk.
@@ -550,22 +554,27 @@ static int score_grad_run(const boac_geom* g, const boac_tissue* t, const float*
                 nxt = temps[next_temp];
                 next_temp ^= 1;
             }
-            mlem_step(cur, nxt, qseg, rseg, zseg);
+            s = mlem_step(cur, nxt, qseg, rseg, zseg);
+            if (s != BOAC_OK) return s;
             cur = nxt;
         }
         if (K == 0) cudaMemcpyAsync(Fk, ck, sizeof(float) * cnt_pix, cudaMemcpyDeviceToDevice, st);
     }
     // ---- score and d L / d q^K
     phase.next("gradient: score and its adjoint");
-    project_table(g, B, tab, Fk, dx, qK, st);
+    s = project_table(g, B, tab, Fk, dx, qK, st);
+    if (s != BOAC_OK) return s;
     const double* lgS = include_lgamma && s_stride == 0
                             ? lgamma_sum((int)vb, S, reinterpret_cast<double*>(base + lay.lg), st)
                             : nullptr;
-    loglik_launch((int)vb, B, qK, S, s_stride, include_lgamma, L, lgS, nullptr, st);
+    s = loglik_launch((int)vb, B, qK, S, s_stride, include_lgamma, L, lgS, nullptr, st);
+    if (s != BOAC_OK) return s;
     if (F_out) cudaMemcpyAsync(F_out, Fk, sizeof(float) * cnt_pix, cudaMemcpyDeviceToDevice, st);
     qbar_final_kernel<<<g1b, 256, 0, st>>>(B, (int)vb, S, s_stride, qK, qbar);
-    backproject_table(g, B, tab, qbar, dx, Fbar, 0, partial, st);
-    abar_accum(g, B, dx, qbar, Fk, nullptr, nullptr, abar, st);
+    s = backproject_table(g, B, tab, qbar, dx, Fbar, 0, partial, st);
+    if (s != BOAC_OK) return s;
+    s = abar_accum(g, B, dx, qbar, Fk, nullptr, nullptr, abar, st);
+    if (s != BOAC_OK) return s;
 
     // ---- reverse through the iterations, one checkpoint segment at a time
     phase.next("gradient: reverse sweep");
@@ -574,9 +583,11 @@ static int score_grad_run(const boac_geom* g, const boac_tissue* t, const float*
         const int n0 = j * ckpt_every;
         const int len = (K - n0) < ckpt_every ? (K - n0) : ckpt_every;
         cudaMemcpyAsync(Fseg, ck + (size_t)j * B * nn, sizeof(float) * cnt_pix, cudaMemcpyDeviceToDevice, st);
-        for (int tt = 0; tt < len; ++tt)
-            mlem_step(Fseg + (size_t)tt * B * nn, Fseg + (size_t)(tt + 1) * B * nn, qseg + (size_t)tt * B * vb,
-                      rseg + (size_t)tt * B * vb, zseg + (size_t)tt * B * nn);
+        for (int tt = 0; tt < len; ++tt) {
+            s = mlem_step(Fseg + (size_t)tt * B * nn, Fseg + (size_t)(tt + 1) * B * nn, qseg + (size_t)tt * B * vb,
+                          rseg + (size_t)tt * B * vb, zseg + (size_t)tt * B * nn);
+            if (s != BOAC_OK) return s;
+        }
         for (int tt = len - 1; tt >= 0; --tt) {
             const float* Fn = Fseg + (size_t)tt * B * nn;
             const float* Fn1 = Fseg + (size_t)(tt + 1) * B * nn;
@@ -584,20 +595,25 @@ static int score_grad_run(const boac_geom* g, const boac_tissue* t, const float*
             const float* r = rseg + (size_t)tt * B * vb;
             const float* z = zseg + (size_t)tt * B * nn;
             mlem_step_adjoint_kernel<<<g1p, 256, 0, st>>>(cnt_pix, Fbar, Fn, Fn1, z, sens, zbar, sensbar, Fnew);
-            project_table(g, B, tab, zbar, dx, rbar, st);
+            s = project_table(g, B, tab, zbar, dx, rbar, st);
+            if (s != BOAC_OK) return s;
             qbar_step_kernel<<<g1b, 256, 0, st>>>(B, (int)vb, S, s_stride, q, rbar, qbar);
-            backproject_table(g, B, tab, qbar, dx, Fnew, 1, partial, st);
-            abar_accum(g, B, dx, r, zbar, qbar, Fn, abar, st);
+            s = backproject_table(g, B, tab, qbar, dx, Fnew, 1, partial, st);
+            if (s != BOAC_OK) return s;
+            s = abar_accum(g, B, dx, r, zbar, qbar, Fn, abar, st);
+            if (s != BOAC_OK) return s;
             float* tmp = Fbar;
             Fbar = Fnew;
             Fnew = tmp;
         }
     }
     // sens = A^T 1
-    abar_accum(g, B, dx, nullptr, sensbar, nullptr, nullptr, abar, st);
+    s = abar_accum(g, B, dx, nullptr, sensbar, nullptr, nullptr, abar, st);
+    if (s != BOAC_OK) return s;
     // attenuation -> mu samples -> pixels -> coefficients
     mbar_kernel<<<rg, kRayThreads, 0, st>>>(n, V, dx, tab, abar);
-    backproject_table(g, B, abar, nullptr, 1.0f, mubar, 0, partial, st);
+    s = backproject_table(g, B, abar, nullptr, 1.0f, mubar, 0, partial, st);
+    if (s != BOAC_OK) return s;
     return coef_launch(g, t, c, mubar, B, reinterpret_cast<double*>(base + lay.coefp), dL_dc, st);
 }
 

@@ -608,14 +608,18 @@ extern "C" int boac_mlem_plain(const boac_geom* g, const float* mu, const float*
         int s = backproject_table(g, 1, tab, nullptr, dx, sens, 0, partial, st);
         if (s != BOAC_OK) return s;
         for (int it = 0; it < K; ++it) {
-            project_table(g, 1, tab, F_c, dx, q, st);
+            s = project_table(g, 1, tab, F_c, dx, q, st);
+            if (s != BOAC_OK) return s;
             ratio_kernel<<<grid_1d((long long)vb, 256), 256, 0, st>>>((int)vb, S_c, q, r);
-            backproject_table(g, 1, tab, r, dx, bp, 0, partial, st);
+            s = backproject_table(g, 1, tab, r, dx, bp, 0, partial, st);
+            if (s != BOAC_OK) return s;
             update_kernel<<<grid_1d((long long)nn, 256), 256, 0, st>>>((int)nn, F_c, bp, sens);
         }
         if (L) {
-            project_table(g, 1, tab, F_c, dx, q, st);
-            loglik_launch((int)vb, 1, q, S_c, 0, include_lgamma, L + cand, nullptr, nullptr, st);
+            s = project_table(g, 1, tab, F_c, dx, q, st);
+            if (s != BOAC_OK) return s;
+            s = loglik_launch((int)vb, 1, q, S_c, 0, include_lgamma, L + cand, nullptr, nullptr, st);
+            if (s != BOAC_OK) return s;
         }
         s = launch_status();
         if (s != BOAC_OK) return s;

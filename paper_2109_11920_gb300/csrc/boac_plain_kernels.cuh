@@ -36,8 +36,10 @@ __global__ void loglik_kernel(int nbin, const float* __restrict__ q, const float
                               long long s_stride, int include_lgamma, double* __restrict__ L,
                               const double* __restrict__ lgS, int* status = nullptr);
 // Launch it for B candidates, on clusters where that is faster (same bits).
-int loglik_launch(int nbin, int B, const float* q, const float* S, long long s_stride, int include_lgamma, double* L,
-                  const double* lgS, int* status, cudaStream_t st);
+// (The launchers below read, and so clear, the CUDA error: the status they
+// return is the only report of a refused launch.)
+[[nodiscard]] int loglik_launch(int nbin, int B, const float* q, const float* S, long long s_stride, int include_lgamma,
+                                double* L, const double* lgS, int* status, cudaStream_t st);
 // sum_i lgamma(S_i + 1) of one sinogram S[nbin] into scratch[0]
 // (scratch: kLgammaScratchDoubles doubles, 8-byte aligned); returns scratch.
 constexpr int kLgammaScratchDoubles = 31;
@@ -58,16 +60,17 @@ size_t bp_partial_floats(const boac_geom* g, int B);
 // q[cand][v][bin] = dx * sum_k tab_v[k][bin] F(sample (k, bin) of view v) for
 // B candidates (boac_bpgroup.cu): one CTA per candidate and sample grid with
 // F in shared memory, or one thread per ray where no grouped kernel exists.
-int project_table(const boac_geom* g, int B, const float* tab, const float* F, float dx, float* q,
-                  cudaStream_t st);
+[[nodiscard]] int project_table(const boac_geom* g, int B, const float* tab, const float* F, float dx, float* q,
+                                cudaStream_t st);
 // One whole MLEM iteration F <- F A^T(S / A F) / sens from the table, for
 // geometries with grouped kernels (mlem_grouped): two launches, `partial` as
 // above, sched from mlem_group_sched (nullptr where none is kept).
 bool mlem_grouped(const boac_geom* g);
 const unsigned short* mlem_group_sched(const boac_geom* g, cudaStream_t st, int* status);
-int mlem_group_iteration(const boac_geom* g, int B, float dx, const float* tab, const float* S, long long s_stride,
-                         float* F, const float* sens, const unsigned short* sched, float* partial, cudaStream_t st);
-int backproject_table(const boac_geom* g, int B, const float* tab, const float* y, float scale, float* out,
-                      int accumulate, float* partial, cudaStream_t st);
+[[nodiscard]] int mlem_group_iteration(const boac_geom* g, int B, float dx, const float* tab, const float* S,
+                                       long long s_stride, float* F, const float* sens, const unsigned short* sched,
+                                       float* partial, cudaStream_t st);
+[[nodiscard]] int backproject_table(const boac_geom* g, int B, const float* tab, const float* y, float scale, float* out,
+                                    int accumulate, float* partial, cudaStream_t st);
 
 }  // namespace boac

@@ -686,7 +686,7 @@ extern "C" int boac_sysmat_mlem(const boac_sysmat* m, const float* vals, const f
                                                                         Fi, B, S, s_stride, r);
         double* scratch = reinterpret_cast<double*>(r + G * (size_t)R * kCandGroup);
         const double* lgS = include_lgamma && s_stride == 0 ? lgamma_sum(R, S, scratch, st) : nullptr;
-        loglik_launch(R, B, r, S, s_stride, include_lgamma, L, lgS, nullptr, st);
+        return loglik_launch(R, B, r, S, s_stride, include_lgamma, L, lgS, nullptr, st);
     }
     return launch_status();
 }
