@@ -411,8 +411,8 @@ __global__ void __launch_bounds__(256) loglik_cluster_kernel(int nbin, int chunk
                                                             const float* __restrict__ S, long long s_stride,
                                                             int include_lgamma, double* __restrict__ L,
                                                             const double* __restrict__ lgS, int* status) {
-    extern __shared__ __align__(16) double terms[];
-    __shared__ double part[32];
+    extern __shared__ __align__(16) double terms[];  // [chunk], then [32] (no static array: see loglik_launch)
+    double* part = terms + chunk;
     cg::cluster_group cl = cg::this_cluster();
     const int ranks = (int)cl.num_blocks(), rank = (int)cl.block_rank(), cand = blockIdx.x / ranks;
     const float* qc = q + (size_t)cand * nbin;
@@ -441,11 +441,14 @@ __global__ void __launch_bounds__(256) loglik_cluster_kernel(int nbin, int chunk
 
 int loglik_launch(int nbin, int B, const float* q, const float* S, long long s_stride, int include_lgamma, double* L,
                   const double* lgS, int* status, cudaStream_t st) {
-    // Eight CTAs per candidate where their terms fit 48 KB each and the batch
-    // leaves SMs idle (one CTA per candidate reaches every SM at 152).
+    // Eight CTAs per candidate where their terms and partial sums fit 48 KB
+    // each, all the shared memory (static arrays included) that a launch gets
+    // without an attribute, and the batch leaves SMs idle (one CTA per
+    // candidate reaches every SM at 152).
     constexpr int kRanks = 8;
     const int chunk = (nbin + kRanks - 1) / kRanks;
-    if (B > 64 || chunk * sizeof(double) > 48 * 1024) {
+    const size_t smem = sizeof(double) * ((size_t)chunk + 32);
+    if (B > 64 || smem > 48 * 1024) {
         loglik_kernel<<<B, 256, 0, st>>>(nbin, q, S, s_stride, include_lgamma, L, lgS, status);
         return launch_status();
     }
@@ -457,7 +460,7 @@ int loglik_launch(int nbin, int B, const float* q, const float* S, long long s_s
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(B * kRanks), 1, 1);
     cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = chunk * sizeof(double);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
