@@ -27,10 +27,11 @@
  *     device.  The library allocates no device memory: operations that need
  *     scratch take a caller-allocated workspace (see boac_workspace_bytes).
  *     It holds two arrays of static device memory on every GPU that loads
- *     it: the 64 MiB scratch of boac_mlem_noalloc and 32 MiB of scatter
- *     schedules kept across calls for up to 8 geometries (the fused kernels
- *     build a geometry's schedule once; later geometries build it in the
- *     workspace on every call).
+ *     it: the 64 MiB scratch of boac_mlem_noalloc and 64 MiB of scatter
+ *     schedules kept across calls (built on a geometry's first call; 60
+ *     geometries of 128 x 128 and 120 views).  A geometry that finds no room,
+ *     or whose schedule is larger than 4 MiB, has it built in the workspace on
+ *     every call, or scatters without one; the results are the same.
  *   - Work is enqueued asynchronously on `stream` (a cudaStream_t; NULL =
  *     the legacy default stream).  Return values report argument and launch
  *     errors only; kernel faults surface at the next synchronisation.
@@ -157,6 +158,18 @@ int boac_test_mlem_handover(const boac_geom *g, const float *mu,
                             const float *S, float *F, int K, int B, double *L,
                             int config, int holders, int withhold, void *ws,
                             size_t ws_bytes, void *stream);
+
+/* ---- test hook of the scatter schedule ----------------------------------
+ * The paper has no counterpart.  Builds the scatter schedule of geometry g
+ * (n = 64, 96 or 128) with `views_per_grid` (2 or 4) views per sample grid,
+ * for a sample buffer of pitch n + pad (pad 1 or 4), into `sched`
+ * (boac_test_schedule_bytes bytes, device): per grid and class
+ * ((k mod 3) * 3 + b mod 3) 16 n entries k << 8 | b, each sample that touches
+ * the image once, 0xFFFF for an empty slot.  Errors: BOAC_EINVAL;
+ * BOAC_EWORKSPACE. */
+size_t boac_test_schedule_bytes(const boac_geom *g, int views_per_grid);
+int boac_test_schedule(const boac_geom *g, int views_per_grid, int pad,
+                       void *sched, size_t bytes, void *stream);
 
 /* Bytes of device workspace that `op` needs for B candidates of geometry g
  * on the current device (0 if none).  For BOAC_OP_SCORE_GRAD the size also

@@ -86,6 +86,8 @@ SIGNATURES = {
     "boac_set_wait_cycles": (_LL, [_LL]),
     "boac_test_mlem_handover_bytes": (_SZ, [_GP, _I, _I, _I, _I]),
     "boac_test_mlem_handover": (_I, [_GP, _P, _P, _P, _I, _I, _P, _I, _I, _I, _P, _SZ, _P]),
+    "boac_test_schedule_bytes": (_SZ, [_GP, _I]),
+    "boac_test_schedule": (_I, [_GP, _I, _I, _P, _SZ, _P]),
     "boac_rasterize_mu": (_I, [_GP, _TP, _P, _I, _I, _P, _P]),
     "boac_rasterize_mu_params": (_I, [_GP, _P, _I, _I, _P, _P]),
     "boac_project": (_I, [_GP, _P, _P, _I, _P, _P]),

@@ -69,6 +69,11 @@ __host__ __device__ constexpr unsigned long long sched_tag_value(int n, int V, i
 // One CTA per (grid, class), for a sample buffer of pitch WP (the W banks of
 // the rounds).  With a tag that already holds `want` (a cached schedule of
 // this geometry and pitch) every CTA returns at once.
+// Two builds on different streams may write one kept schedule at the same
+// time, and one stream's kernel may read it while the other's builder still
+// writes.  So the entries depend on the geometry and the pitch alone (no order
+// of arrival), they are worked out in shared memory, and each is stored once:
+// every store writes the value that is there already or will be.
 template <int N, int WP>
 __global__ void __launch_bounds__(256) scatter_schedule_kernel(int V, unsigned short* __restrict__ sched,
                                                                const unsigned long long* tag,
@@ -81,8 +86,8 @@ __global__ void __launch_bounds__(256) scatter_schedule_kernel(int V, unsigned s
     const int nbc = (N - pb + 2) / 3, cnt = ((N - pk + 2) / 3) * nbc;
     __shared__ unsigned short ent[S::CLS_MAX];  // samples grouped by (bank, W bank)
     __shared__ unsigned short key[S::CLS_MAX];  // (bank << 5 | W bank) of sample t, or empty
+    __shared__ __align__(4) unsigned short slot[S::CLS_ENTRIES];  // the class's entries
     __shared__ int num[1024], start[1024], cur[1024];
-    __shared__ int s_rounds;
     float cs, sn;
     cta_view_cos_sin(gi, V, &cs, &sn);  // grid gi's base view, as in the fused kernel
     const float c = 0.5f * (float)(N - 1);
@@ -124,6 +129,19 @@ __global__ void __launch_bounds__(256) scatter_schedule_kernel(int V, unsigned s
         if (kk != kSchedEmpty)
             ent[atomicAdd(&cur[kk], 1)] = (unsigned short)(((pk + 3 * (t / nbc)) << 8) | (pb + 3 * (t % nbc)));
     }
+    for (int t = threadIdx.x; t < S::CLS_ENTRIES; t += blockDim.x) slot[t] = kSchedEmpty;
+    __syncthreads();
+    // A cell's samples in ascending order, not in the order in which the
+    // atomics above let them arrive.
+    for (int cell = threadIdx.x; cell < 1024; cell += blockDim.x) {
+        unsigned short* e = ent + start[cell];
+        for (int i = 1; i < num[cell]; ++i) {
+            const unsigned short x = e[i];
+            int j = i;
+            for (; j > 0 && e[j - 1] > x; --j) e[j] = e[j - 1];
+            e[j] = x;
+        }
+    }
     __syncthreads();
     if (threadIdx.x < 32) {
         int r = 0;
@@ -160,12 +178,13 @@ __global__ void __launch_bounds__(256) scatter_schedule_kernel(int V, unsigned s
                     --left;
                 }
             }
-            out[sched_slot(r, lane)] = pick >= 0 ? (unsigned short)pick : kSchedEmpty;
+            if (pick >= 0) slot[sched_slot(r, lane)] = (unsigned short)pick;
             ++r;
         }
         // Samples left after the last round's capacity: into the empty slots
         // of their accumulator bank (only the sample buffer's banks may then
-        // clash), and those that find none into any empty slot.
+        // clash), and those that find none into any empty slot (a class has
+        // at most CLS_MAX <= CLS_ENTRIES samples: there is one for each).
         if (__any_sync(0xffffffffu, left > 0)) {
             __syncwarp();
             int cell = lane * 32;
@@ -174,8 +193,8 @@ __global__ void __launch_bounds__(256) scatter_schedule_kernel(int V, unsigned s
                 return ent[start[cell] + cur[cell]++];
             };
             for (int q = 0; q < r && left > 0; ++q)
-                if (out[sched_slot(q, lane)] == kSchedEmpty) {
-                    out[sched_slot(q, lane)] = take();
+                if (slot[sched_slot(q, lane)] == kSchedEmpty) {
+                    slot[sched_slot(q, lane)] = take();
                     --left;
                 }
             int at = 0;
@@ -183,18 +202,18 @@ __global__ void __launch_bounds__(256) scatter_schedule_kernel(int V, unsigned s
                 __syncwarp();
                 if (lane == l)
                     for (; left > 0; --left) {
-                        while (out[sched_slot(at >> 5, at & 31)] != kSchedEmpty) ++at;
-                        out[sched_slot(at >> 5, at & 31)] = take();
+                        while (at < S::CLS_ENTRIES && slot[sched_slot(at >> 5, at & 31)] != kSchedEmpty) ++at;
+                        if (at == S::CLS_ENTRIES) break;
+                        slot[sched_slot(at >> 5, at & 31)] = take();
                     }
                 at = __shfl_sync(0xffffffffu, at, l);
             }
         }
-        if (lane == 0) s_rounds = r;
     }
     __syncthreads();
-    // the slots after the last round
-    for (int t = 32 * s_rounds + threadIdx.x; t < S::CLS_ENTRIES; t += blockDim.x)
-        out[sched_slot(t / 32, t % 32)] = kSchedEmpty;
+    // every entry once, two to a word
+    for (int t = threadIdx.x; t < S::CLS_WORDS; t += blockDim.x)
+        reinterpret_cast<unsigned*>(out)[t] = reinterpret_cast<const unsigned*>(slot)[t];
 }
 
 // Launch the schedule builder for images up to 128 x 128 and a sample

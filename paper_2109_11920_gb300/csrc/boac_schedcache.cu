@@ -15,7 +15,8 @@
 // return at once when the tag already names the geometry, then a one-thread
 // kernel that writes the tag (after the build, in stream order).  Two calls
 // on different streams that both find the tag empty build the schedule at the
-// same time and write the same values.
+// same time and store the same bytes (scatter_schedule_kernel), so neither a
+// kernel that reads it meanwhile nor a later one sees anything else.
 //
 // A geometry that finds no room, or whose schedule is larger than 4 MiB, has
 // no kept schedule: it is built into the caller's workspace on every call, or,
@@ -35,7 +36,7 @@ namespace boac {
 namespace {
 
 constexpr int kSchedCacheSlots = 256;
-constexpr size_t kSchedArenaEntries = ((size_t)64 << 20) / sizeof(unsigned short);  // 58 of 1.1 MB (128 x 128, 120 views)
+constexpr size_t kSchedArenaEntries = ((size_t)64 << 20) / sizeof(unsigned short);  // 60 of 1.1 MB (128 x 128, 120 views)
 constexpr size_t kSchedMaxBytes = (size_t)4 << 20;  // the largest schedule kept
 constexpr int kSchedCacheDevices = 64;
 
@@ -105,3 +106,22 @@ const unsigned short* sched_prepare(int n, int V, int ngrid, int wp, unsigned sh
 }
 
 }  // namespace boac
+
+using namespace boac;
+
+// Test hook: the schedule that the library builds for g and a sample buffer of
+// pitch n + pad, into the caller's memory.
+extern "C" size_t boac_test_schedule_bytes(const boac_geom* g, int views_per_grid) {
+    if (!geom_ok(g) || (g->n != 64 && g->n != 96 && g->n != 128)) return 0;
+    if ((views_per_grid != 2 && views_per_grid != 4) || g->n_views % views_per_grid) return 0;
+    return sched_bytes(g->n, g->n_views / views_per_grid);
+}
+
+extern "C" int boac_test_schedule(const boac_geom* g, int views_per_grid, int pad, void* sched, size_t bytes,
+                                  void* stream) {
+    const size_t need = boac_test_schedule_bytes(g, views_per_grid);
+    if (need == 0 || !sched || (pad != 1 && pad != 4)) return BOAC_EINVAL;
+    if (bytes < need) return BOAC_EWORKSPACE;
+    return sched_launch(g->n, g->n_views, g->n_views / views_per_grid, g->n + pad, static_cast<unsigned short*>(sched),
+                        as_stream(stream));
+}
