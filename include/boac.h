@@ -119,15 +119,16 @@ int boac_bounds_faults(int *faults, int reset);
  * -inf in L, not a failure).  boac_mlem_plain, boac_score and boac_loglik
  * keep no status word: there the -inf in L is the only report.  The fused kernel splits the batch's iterations evenly over
  * its CTAs, so a candidate may be continued by a second CTA, which waits for
- * a flag from the first; the schedule leaves that wait a whole candidate's
- * worth of slack, and it gives up after a limit set by boac_set_wait_cycles
- * (default about 2 s).  Synchronous: copies the
- * word to *status after the device work queued before it has finished. */
+ * a flag from the first and gives up when the first part takes longer than
+ * its iterations can account for (as timed by the second part's set-up) by a
+ * limit set by boac_set_wait_cycles (default about 2 s).  Synchronous: copies
+ * the word to *status after the device work queued before it has finished. */
 int boac_workspace_status(const void *ws, size_t ws_bytes, int *status);
 
 /* Limit, in GPU clock cycles, of the bounded hand-over wait described above
  * (the second part of a cut candidate waiting for the first part's flag),
- * for every launch that follows, process-wide.  cycles <= 0 restores the
+ * beyond the time that the first part may take, for every launch that
+ * follows, process-wide.  cycles <= 0 restores the
  * default, 2^32 (about 2 s at 2 GHz).  Returns the previous limit.  A
  * shorter limit gives up sooner on a GPU shared with other work, where a
  * CTA of the launch may wait for an SM; a longer one tolerates more such

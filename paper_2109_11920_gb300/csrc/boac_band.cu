@@ -349,6 +349,7 @@ __global__ void __launch_bounds__(4 * N, N == 64 ? 4 : (N == 128 && NB > 2) ? 2 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* dred = reinterpret_cast<double*>(smem_raw);
     int* flag = reinterpret_cast<int*>(smem_raw + 32 * sizeof(double));  // [0]: hand-over
+    long long* t_begin = reinterpret_cast<long long*>(flag + 2);         // the clock at the candidate's start
     float* sm = reinterpret_cast<float*>(smem_raw + L::HEAD);
     int* recs = reinterpret_cast<int*>(smem_raw + L::RECS);  // [2][REC]
     float* Fb = sm + L::F0;
@@ -450,6 +451,7 @@ __global__ void __launch_bounds__(4 * N, N == 64 ? 4 : (N == 128 && NB > 2) ? 2 
         const int it0 = (int)(u0 < Kc ? u0 : Kc), it1 = (int)(u1 < Kc ? u1 : Kc);
 
         // ---- set-up: mu band -> Fb, accumulator cleared
+        if (tid == 0) *t_begin = clock64();
         for (int i = tid; i < BIMG; i += NT) {
             Fb[i] = 0.0f;
             Ab[i] = 0.0f;
@@ -589,12 +591,12 @@ __global__ void __launch_bounds__(4 * N, N == 64 ? 4 : (N == 128 && NB > 2) ? 2 
         if (r == 0 && tid == 0) {
             int ok = 1;
             if (!first) {
-                const long long t0 = clock64();
+                const long long t0 = clock64(), limit = wait_limit(a, u0, t0 - *t_begin);
                 for (;;) {
                     int f;
                     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(f) : "l"(a.ready + cand) : "memory");
                     if (f) break;
-                    if (clock64() - t0 > a.wait_cycles) {
+                    if (clock64() - t0 > limit) {
                         ok = 0;
                         atomicExch(a.status, BOAC_ETIMEOUT);
                         break;

@@ -48,14 +48,18 @@ struct FusedArgs {
     // gets the same share, a candidate is cut between at most two CTAs).
     // A CTA takes its candidates in descending order, so the first part of
     // a cut candidate runs first on CTA m and its second part last on CTA
-    // m+1; ready[j] tells the second part that the first has written F
-    // (always long before it is needed, since cap >= the candidate length).
+    // m+1; ready[j] tells the second part that the first has written F.  Where
+    // CTA m + 1 has cap units and is no faster than CTA m, that is before it
+    // is needed (cap >= the candidate length).  The last CTA has fewer units,
+    // and in a ragged batch whose classes share the SMs one CTA may be slower
+    // than another: the second part then waits (wait_limit).
     const long long* job_start;
     long long cap;
     int* ready;    // [B] zeroed before the launch
     int* status;   // 0, or BOAC_ETIMEOUT if a bounded wait ran out
     // Cycles the second part of a cut candidate waits for the first part's
-    // flag before giving up (boac_set_wait_cycles; default kWaitCycles).
+    // flag beyond the time that part may take (wait_limit) before giving up
+    // (boac_set_wait_cycles; default kWaitCycles).
     long long wait_cycles;
     // Candidate whose first part does not release its flag (-1: none).  Set
     // only by boac_test_mlem_handover, to make the bounded wait run out.
@@ -87,6 +91,16 @@ __device__ __forceinline__ void class_end(const FusedArgs& a) {
     __syncthreads();
     if (threadIdx.x == 0 && atomicAdd(a.done, 1) == (int)gridDim.x - 1)
         asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// The hand-over wait's limit, for a second part that set its candidate up in
+// `setup` cycles and whose first part is u0 iterations: set-up takes about as
+// long as 1.7 iterations on the same CTA (128 x 128, 120 views; 1.05 M against
+// 0.62 M cycles), and CTAs that share an SM take up to 1.9 times the time of
+// one alone, so four set-ups per iteration of the first part allow for it
+// however long the candidate is.  (The first part's CTA starts no later: CTAs
+// are dispatched in index order.)
+__device__ __forceinline__ long long wait_limit(const FusedArgs& a, long long u0, long long setup) {
+    return a.wait_cycles + 4 * u0 * setup;
 }
 // Element i of every rank's copy of a shared-memory array, summed in rank
 // order; and the same value stored into every rank's copy.  All the loads are
@@ -123,9 +137,7 @@ inline void overlap_attribute(cudaLaunchAttribute* attr, const FusedArgs& a) {
     attr->val.programmaticStreamSerializationAllowed = (a.overlap & FusedArgs::kJoin) ? 1 : 0;
 }
 
-// Default number of cycles a CTA waits for the first part of a cut candidate
-// before giving up (about 2 s at 2 GHz; the schedule leaves the wait a whole
-// candidate's worth of slack, so it ends immediately in practice).
+// Default of wait_cycles: about 2 s at 2 GHz.
 constexpr long long kWaitCycles = 1LL << 32;
 // The process-wide wait limit in force (boac_set_wait_cycles).
 long long wait_cycles();

@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
     }
 
     __shared__ int wait_ok;
+    __shared__ long long t_begin;  // the clock at the candidate's start
     const long long units = a.job_start ? a.job_start[a.B] : (long long)a.B * (a.K > 0 ? a.K : 1);
     const long long m0 = (long long)blockIdx.x * a.cap;
     const long long m1 = m0 + a.cap < units ? m0 + a.cap : units;
@@ -273,6 +274,7 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
         const int it0 = (int)(u0 < Kc ? u0 : Kc), it1 = (int)(u1 < Kc ? u1 : Kc);
 
         // ---- set-up: mu -> img0 (zero ring), img1 = 0
+        if (tid == 0) t_begin = clock64();
         for (int i = tid; i < IMG; i += NT) {
             img0[i] = 0.0f;
             img1[i] = 0.0f;
@@ -383,12 +385,12 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
         if (tid == 0) {  // second part of a cut candidate: wait for the first
             int ok = 1;
             if (!first) {
-                const long long t0 = clock64();
+                const long long t0 = clock64(), limit = wait_limit(a, u0, t0 - t_begin);
                 for (;;) {
                     int f;
                     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(f) : "l"(a.ready + cand) : "memory");
                     if (f) break;
-                    if (clock64() - t0 > a.wait_cycles) {
+                    if (clock64() - t0 > limit) {
                         ok = 0;
                         atomicExch(a.status, BOAC_ETIMEOUT);
                         break;
