@@ -85,7 +85,7 @@ template <int N, int NT, bool QUAD>
 static FusedVariant make_variant() {
     return FusedVariant{N, NT, QUAD, 1, smem_of<N, NT>, (const void*)mlem_fused_kernel<N, NT, QUAD>,
                         fused_prepare_t<N, NT, QUAD>, fused_launch_t<N, NT, QUAD>, 1, nullptr,
-                        fused_image_floats<N, NT>()};
+                        fused_image_floats<N, NT>(), fused_tmem_columns<N, NT, QUAD>()};
 }
 
 template <int N, int NB>
@@ -101,7 +101,7 @@ static int band_launch_of(const FusedArgs& a, int clusters, cudaStream_t st) {
 template <int N, int NB>
 static FusedVariant make_band_variant() {
     return FusedVariant{N, 4 * N, true, NB, band_smem_of<N, NB>, nullptr, band_prepare_of<N, NB>,
-                        band_launch_of<N, NB>, 1, nullptr, 0};
+                        band_launch_of<N, NB>, 1, nullptr, 0, 0};
 }
 
 #define BOAC_SHAPES(NV)                                                                        \
@@ -236,6 +236,29 @@ static const FusedVariant* get_variant(const boac_geom* g, int config) {
     return v;
 }
 
+// CTAs of a kernel that fit an SM by registers (given out in units of 8 per
+// thread to the warps of the SM's four parts), shared memory, threads and
+// columns of tensor memory; 0 after an error.  The runtime's occupancy query
+// answers 1 for every kernel that allocates tensor memory, whatever its size,
+// while the SM holds as many as fit: taken at its word it left 64 x 64 batches
+// of more than one candidate per SM with one CTA on each (20 iterations: 456
+// candidates of 60 views 5.44 -> 3.32 ms, 1000 12.13 -> 7.37, 456 of 90 views
+// 17.7 -> 8.9).
+static int resident_ctas(const FusedVariant* v, int dev) {
+    cudaFuncAttributes fa;
+    int regs = 0, smem = 0, reserved = 0, threads = 0;
+    if (cudaFuncGetAttributes(&fa, v->func) != cudaSuccess ||
+        cudaDeviceGetAttribute(&regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev) != cudaSuccess)
+        return 0;
+    const int warps = (v->nt + 31) / 32, per_warp = (fa.numRegs + 7) / 8 * 8 * 32;
+    const int by_regs = 4 * (regs / 4 / per_warp) / warps;
+    const int by_smem = (int)(smem / (v->smem(kMaxViews) + fa.sharedSizeBytes + reserved));
+    return std::min({by_regs, by_smem, threads / v->nt, kTmemColumns / v->tmem_cols});
+}
+
 // Resident CTAs per SM of a variant, computed for the largest view table it
 // may be launched with (the per-view table is a few KB, so this equals the
 // occupancy at every view count); cached per device.
@@ -257,8 +280,10 @@ static int variant_occupancy(const FusedVariant* v, int V) {
         return 0;
     }
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, v->func, v->nt, v->smem(kMaxViews)) !=
-        cudaSuccess) {
+    if (v->tmem_cols > 0) nb = resident_ctas(v, dev);
+    else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, v->func, v->nt, v->smem(kMaxViews)) != cudaSuccess)
+        nb = 0;
+    if (nb <= 0) {
         cudaGetLastError();
         return 0;
     }
@@ -303,7 +328,12 @@ static FusedLayout fused_layout(const boac_geom* g, const FusedVariant* v, int h
     return l;
 }
 
-// CTAs (one-CTA kernel) or clusters that run at once, at most B.
+// CTAs (one-CTA kernel) or clusters that run at once, at most B.  Where several
+// 64 x 64 CTAs fit an SM, a second one takes the two 1.6 times the time of one
+// (two views per grid 1.4 times): up to that many candidates per SM, one CTA on
+// each with an even split ends sooner than a whole candidate per CTA (60 views,
+// 20 iterations: 160 candidates 1.66 against 2.24 ms, 200 2.06 against 2.25, 304
+// 2.75 against 2.28; 90 views: 160 5.09 against 6.08, 200 6.16 against 6.10).
 static int variant_holders(const boac_geom* g, const FusedVariant* v, int B) {
     long long h;
     if (v->nb > 1) {
@@ -313,6 +343,7 @@ static int variant_holders(const boac_geom* g, const FusedVariant* v, int B) {
     } else {
         const int per_sm = variant_occupancy(v, g->n_views);
         h = (long long)per_sm * sm_count();
+        if (per_sm > 1 && B > sm_count() && 10LL * B < (v->quad ? 16LL : 14LL) * sm_count()) h = sm_count();
     }
     if (h <= 0) return 0;
     return (int)(h < B ? h : B);

@@ -97,6 +97,18 @@ constexpr int fused_min_blocks() {
     return (N <= 64 ? 3 : 1) < 1024 / NT ? (N <= 64 ? 3 : 1) : (1024 / NT > 0 ? 1024 / NT : 1);
 }
 
+// Tensor memory of a CTA (see the kernel): floats per thread, and the columns
+// they take; 0 where they are more than an SM has and nothing is kept there.
+template <int N, int NT, bool QUAD>
+constexpr int fused_stash() {
+    return (QUAD ? 4 : 2) * FusedShape<N, NT>::SEG;
+}
+template <int N, int NT, bool QUAD>
+constexpr int fused_tmem_columns() {
+    constexpr int c = tmem_columns(NT / 32, fused_stash<N, NT, QUAD>());
+    return c <= kTmemColumns ? c : 0;
+}
+
 // A thread's exponents of one grid, from the workspace planes into tensor
 // memory: chunk i is four samples of its column run, or (i >= SEG / 4) of its
 // row run.  A run's exponents lie in the upper half of the columns that its
@@ -199,8 +211,8 @@ __global__ void __launch_bounds__(NT, (G > 1 ? 1 : fused_min_blocks<N, NT>())) m
     // 256 x 256 images (four times the samples per thread) do not fit and
     // read the exponents twice.  CTAs that share an SM (64 x 64 only, at most
     // three by shared memory) take 128 columns each.
-    constexpr int kStash = (QUAD ? 4 : 2) * SEG, kTmemCols = tmem_columns(NT / 32, kStash);
-    constexpr bool kStashed = kTmemCols <= 512;
+    constexpr int kStash = fused_stash<N, NT, QUAD>(), kTmemCols = fused_tmem_columns<N, NT, QUAD>();
+    constexpr bool kStashed = kTmemCols > 0;
     __shared__ unsigned tmem_addr;
     unsigned stash = 0;
     if constexpr (kStashed) {
@@ -688,6 +700,7 @@ struct FusedVariant {
     int g;   // CTAs per candidate in the fused kernel's cluster mode (1 otherwise)
     int (*max_clusters)();  // cluster mode: clusters resident at once
     size_t image_floats;    // one-CTA kernel: F, accumulator and sample buffer of a CTA
+    int tmem_cols;          // columns of tensor memory of a CTA (0: none)
 };
 
 template <int N, int NT, bool QUAD>

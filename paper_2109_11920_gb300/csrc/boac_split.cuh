@@ -84,7 +84,7 @@ template <int N, int G>
 static FusedVariant make_split_variant() {
     return FusedVariant{N, 8 * N, true, 1, smem_of<N, 8 * N>, (const void*)mlem_fused_kernel<N, 8 * N, true, G>,
                         fused_prepare_t<N, 8 * N, true>, split_launch_t<N, 8 * N, G>, G, split_max_clusters_t<N, 8 * N, G>,
-                        fused_image_floats<N, 8 * N>()};
+                        fused_image_floats<N, 8 * N>(), fused_tmem_columns<N, 8 * N, true>()};
 }
 
 // The cluster sizes of split_variants (configuration ids 9 ..).

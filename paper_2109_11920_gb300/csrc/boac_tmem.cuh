@@ -14,6 +14,8 @@
 
 namespace boac {
 
+constexpr int kTmemColumns = 512;  // of an SM
+
 // Columns to allocate for a CTA of `warps` warps with `per_thread` floats per
 // thread: a power of two, at least 32.
 __host__ __device__ constexpr int tmem_columns(int warps, int per_thread) {
@@ -27,7 +29,7 @@ __host__ __device__ constexpr int tmem_columns(int warps, int per_thread) {
 // another CTA of the SM holds them) and leaves the address in *smem_addr.
 template <int COLS>
 __device__ __forceinline__ void tmem_alloc(unsigned* smem_addr) {
-    static_assert(COLS >= 32 && COLS <= 512 && (COLS & (COLS - 1)) == 0, "tensor-memory columns");
+    static_assert(COLS >= 32 && COLS <= kTmemColumns && (COLS & (COLS - 1)) == 0, "tensor-memory columns");
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem_addr);
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s), "n"(COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
