@@ -432,6 +432,7 @@ struct RaggedPlan {
     long long units[kMaxRaggedClasses], longest[kMaxRaggedClasses];
     double chain[kMaxRaggedClasses];  // modelled time of the class's busiest CTA
     bool shares_sm[kMaxRaggedClasses];  // several of the class's CTAs fit an SM
+    bool alone[kMaxRaggedClasses];      // the class's kernel runs before the others, on the whole GPU
     int slots[kMaxRaggedClasses];
     const FusedVariant* var[kMaxRaggedClasses];
     size_t desc_off[kMaxRaggedClasses], start_off[kMaxRaggedClasses], layout_off[kMaxRaggedClasses];
@@ -445,8 +446,22 @@ struct RaggedPlan {
 // classes fit the GPU together.  Time per sample grid, measured: 11.1 us at
 // 128 x 128 and 5.3 us at 64 x 64, that is 0.47 ns per sample and as much as
 // 7200 samples for its barriers; two views per grid 0.85 times that (6.5 us
-// at 96 x 96); two CTAs on an SM take 1.45 times the time of one.  A split
-// only decides which CTA runs which iterations, never what they compute.
+// at 96 x 96); a second and third CTA on an SM count as 0.45 of one each.  (They
+// take 0.6 and 0.75: 64 x 64, 60 views, 20 iterations of 152, 304 and 456
+// candidates 1.41, 2.28 and 3.32 ms.  With 0.65, batches take longer: 600 beside
+// 152 of 128 x 128 13.6 against 12.6 ms, 128 beside 128 8.8 against 7.3.)
+//
+// The one-CTA kernel at 256 x 256 keeps its images in global memory and slows
+// down with the CTAs that share L2: 200, 339 and 521 us per grid of two views
+// with 8, 64 and 152 of them, 6.6 times the time of a kernel with its images on
+// chip and 0.085 more per CTA.  Up to kSharedGlobalCtas such CTAs run beside
+// the other classes (32 candidates of 90 views and 16 of 180: 118 ms, one class
+// after the other 129); more of them run first, alone, since they and the others
+// then take each other's L2 (64 beside 152 of 128 x 128: 135 ms, one after the
+// other 111).
+//
+// A split only decides which CTA runs which iterations, never what they compute.
+constexpr int kSharedGlobalCtas = 32;
 static void ragged_share(const boac_geom* classes, int n_classes, RaggedPlan* pl) {
     const int sms = sm_count();
     double cost[kMaxRaggedClasses], T = 0.0, work = 0.0;
@@ -457,9 +472,12 @@ static void ragged_share(const boac_geom* classes, int n_classes, RaggedPlan* pl
         per_sm[c] = v->nb > 1 || v->g > 1 ? 0 : variant_occupancy(v, g.n_views);
         cost[c] = (v->quad ? g.n_views / 4 : 0.85 * (g.n_views / 2)) * ((double)g.n * g.n + 7200.0) *
                   (per_sm[c] > 1 ? 1.0 + 0.45 * (per_sm[c] - 1) : 1.0);
+        const bool global = per_sm[c] > 0 && fused_global_images(g.n);
+        if (global) cost[c] *= 6.6 + 0.085 * pl->slots[c];
+        pl->alone[c] = global && pl->slots[c] > kSharedGlobalCtas;
         pl->chain[c] = 0.0;
         pl->shares_sm[c] = per_sm[c] > 1;
-        if (pl->cls_count[c] == 0) continue;
+        if (pl->cls_count[c] == 0 || pl->alone[c]) continue;
         ++classes_in_use;
         const int ctas = v->nb > 1 ? v->nb : v->g;
         pl->chain[c] = cost[c] / ctas * split_cap(pl->units[c], pl->longest[c], pl->slots[c]);
@@ -473,7 +491,7 @@ static void ragged_share(const boac_geom* classes, int n_classes, RaggedPlan* pl
         int need[kMaxRaggedClasses], used = 0;
         for (int c = 0; c < n_classes; ++c) {
             need[c] = 0;
-            if (pl->cls_count[c] == 0 || per_sm[c] == 0) continue;
+            if (pl->cls_count[c] == 0 || per_sm[c] == 0 || pl->alone[c]) continue;
             const double n = ceil(pl->units[c] * cost[c] / T);
             need[c] = n < pl->slots[c] ? (int)n : pl->slots[c];
             used += (need[c] + per_sm[c] - 1) / per_sm[c];
@@ -677,7 +695,7 @@ extern "C" int boac_mlem_ragged_run(const boac_geom* classes, int n_classes,
     cudaStream_t st = as_stream(stream);
     if (cudaMemsetAsync(base, 0, sizeof(int), st) != cudaSuccess) return launch_status();
     // What every class's kernel needs first, then the kernels, each free to
-    // start beside the ones before it: one after the other they take the sum
+    // start beside the ones before it (but see RaggedPlan::alone): one after the other they take the sum
     // of the classes' longest chains (256 candidates of three sizes, 20 to 80
     // iterations: 57.0 ms, together 28.8).  The longest chain goes first, but
     // CTAs that share an SM last: on an empty GPU each would be given an SM of
@@ -689,6 +707,7 @@ extern "C" int boac_mlem_ragged_run(const boac_geom* classes, int n_classes,
         if (cnt == 0) continue;
         int at = used++;
         auto before = [&](int x, int y) {
+            if (pl.alone[x] != pl.alone[y]) return pl.alone[x];
             return pl.shares_sm[x] != pl.shares_sm[y] ? pl.shares_sm[y] : pl.chain[x] > pl.chain[y];
         };
         for (; at > 0 && before(c, order[at - 1]); --at) order[at] = order[at - 1];
@@ -709,7 +728,9 @@ extern "C" int boac_mlem_ragged_run(const boac_geom* classes, int n_classes,
     }
     for (int i = 0; i < used; ++i) {
         const int c = order[i];
-        args[c].overlap = (i + 1 < used ? FusedArgs::kTrigger : 0) | (i > 0 ? FusedArgs::kJoin : 0);
+        args[c].overlap = pl.alone[c] ? 0
+                                      : (i + 1 < used ? FusedArgs::kTrigger : 0) |
+                                            (i > 0 && !pl.alone[order[i - 1]] ? FusedArgs::kJoin : 0);
         s = pl.var[c]->launch(args[c], grids[c], st);
         if (s != BOAC_OK) return s;
     }

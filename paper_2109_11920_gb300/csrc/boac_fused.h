@@ -95,7 +95,7 @@ __device__ __forceinline__ void class_end(const FusedArgs& a) {
 // The hand-over wait's limit, for a second part that set its candidate up in
 // `setup` cycles and whose first part is u0 iterations: set-up takes about as
 // long as 1.7 iterations on the same CTA (128 x 128, 120 views; 1.05 M against
-// 0.62 M cycles), and CTAs that share an SM take up to 1.9 times the time of
+// 0.62 M cycles), and CTAs that share an SM take up to 2.4 times the time of
 // one alone, so four set-ups per iteration of the first part allow for it
 // however long the candidate is.  (The first part's CTA starts no later: CTAs
 // are dispatched in index order.)
