@@ -364,7 +364,8 @@ int boac_mlem_noalloc(const boac_geom *g, const float *mu, const float *S,
 
 /* ---- Eq. 5: score of given images ---------------------------------------
  * L[b] = sum_i S_i ln q_i - q_i [- ln S_i!], q = A^mu F (float32 projection,
- * float64 reduction; same conventions as boac_mlem).
+ * float64 reduction; same conventions as boac_mlem): boac_loglik of
+ * boac_project's q, bit for bit.
  *   ws  boac_workspace_bytes(g, B, BOAC_OP_SCORE) bytes (holds q). */
 int boac_score(const boac_geom *g, const float *mu, const float *S,
                long long s_stride, const float *F, int B, int include_lgamma,

@@ -576,8 +576,7 @@ extern "C" int boac_score(const boac_geom* g, const float* mu, const float* S, l
     const size_t vb = (size_t)g->n_views * g->n_bins;
     if (!ws || ws_bytes < sizeof(float) * vb * B) return BOAC_EWORKSPACE;
     float* q = static_cast<float*>(ws);
-    project_rays(g, B, mu, F, q, as_stream(stream));
-    int s = launch_status();
+    int s = boac_project(g, mu, F, B, q, stream);
     if (s != BOAC_OK) return s;
     return boac_loglik(g, q, S, s_stride, B, include_lgamma, L, stream);
 }
