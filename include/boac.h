@@ -222,7 +222,11 @@ int boac_project(const boac_geom *g, const float *mu, const float *F, int B,
  *   out [B][n][n]            output (device, float32)
  *   ws  workspace of boac_workspace_bytes(g, B, BOAC_OP_BACKPROJECT) bytes
  *       (holds partial images and, for sizes without the scatter, the
- *       attenuation factors of every ray sample). */
+ *       attenuation factors of every ray sample; the size counts both for
+ *       every geometry).  With less, down to one candidate's and 512 bytes,
+ *       the candidates are done in runs that fit.  How many run at once
+ *       decides how many grids a partial image sums, so where the scatter runs
+ *       B and ws_bytes change an image's rounding (boac_project's not). */
 int boac_backproject(const boac_geom *g, const float *mu, const float *y,
                      int B, float *out, void *ws, size_t ws_bytes,
                      void *stream);
