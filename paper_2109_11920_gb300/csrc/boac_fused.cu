@@ -328,12 +328,7 @@ static FusedLayout fused_layout(const boac_geom* g, const FusedVariant* v, int h
     return l;
 }
 
-// CTAs (one-CTA kernel) or clusters that run at once, at most B.  Where several
-// 64 x 64 CTAs fit an SM, a second one takes the two 1.6 times the time of one
-// (two views per grid 1.4 times): up to that many candidates per SM, one CTA on
-// each with an even split ends sooner than a whole candidate per CTA (60 views,
-// 20 iterations: 160 candidates 1.66 against 2.24 ms, 200 2.06 against 2.25, 304
-// 2.75 against 2.28; 90 views: 160 5.09 against 6.08, 200 6.16 against 6.10).
+// CTAs (one-CTA kernel) or clusters that run at once, at most B.
 static int variant_holders(const boac_geom* g, const FusedVariant* v, int B) {
     long long h;
     if (v->nb > 1) {
@@ -343,10 +338,23 @@ static int variant_holders(const boac_geom* g, const FusedVariant* v, int B) {
     } else {
         const int per_sm = variant_occupancy(v, g->n_views);
         h = (long long)per_sm * sm_count();
-        if (per_sm > 1 && B > sm_count() && 10LL * B < (v->quad ? 16LL : 14LL) * sm_count()) h = sm_count();
     }
     if (h <= 0) return 0;
     return (int)(h < B ? h : B);
+}
+
+// Of them, those that a batch of B candidates with K iterations each is split
+// over.  Where several 64 x 64 CTAs fit an SM, a second one takes the two r = 1.6
+// times the time of one (two views per grid r = 1.4), so a whole candidate per
+// CTA takes r (K + s), s iterations' time for set-up and score; one CTA per SM
+// with an even split takes K B / SMs, and 2.5 iterations more than r s for its
+// second and third candidates: the shorter of the two.  (60 views, 160 and 200
+// candidates: 20 iterations 1.66 and 2.06 against 2.24 and 2.25 ms, one
+// iteration 0.46 and 0.46 against 0.36 and 0.37.)
+static int split_holders(const boac_geom* g, const FusedVariant* v, int B, long long K) {
+    const int h = variant_holders(g, v, B), sms = sm_count();
+    if (v->nb > 1 || v->g > 1 || sms <= 0 || h <= sms) return h;
+    return ((v->quad ? 1.6 : 1.4) - (double)B / sms) * K > 2.5 ? sms : h;
 }
 
 size_t fused_workspace_bytes(const boac_geom* g, int B) {
@@ -530,7 +538,7 @@ static int ragged_plan(const boac_geom* classes, int n_classes, const boac_ragge
         pl->var[c] = get_variant(&classes[c], cfg);
         if (!pl->var[c]) return BOAC_EINVAL;
         const int cnt = pl->cls_count[c];
-        pl->slots[c] = cnt ? variant_holders(&classes[c], pl->var[c], cnt) : 0;
+        pl->slots[c] = cnt ? split_holders(&classes[c], pl->var[c], cnt, pl->units[c] / cnt) : 0;
         if (cnt && pl->slots[c] <= 0) return BOAC_ECUDA;
     }
     ragged_share(classes, n_classes, pl);
@@ -580,7 +588,7 @@ extern "C" int boac_mlem(const boac_geom* g, const float* mu, const float* S, lo
     const int slots = variant_holders(g, v, B);
     if (slots <= 0) return BOAC_ECUDA;
     if (!ws || ws_bytes < fused_layout(g, v, slots, B).total) return BOAC_EWORKSPACE;
-    return launch_uniform(g, v, slots, mu, S, s_stride, F, K, B, L, include_lgamma,
+    return launch_uniform(g, v, split_holders(g, v, B, K), mu, S, s_stride, F, K, B, L, include_lgamma,
                           static_cast<char*>(ws), as_stream(stream));
 }
 
@@ -807,8 +815,9 @@ extern "C" int boac_mlem_noalloc(const boac_geom* g, const float* mu, const floa
     const FusedVariant* v = get_variant(g, single_cta_config(g));
     if (!v) return BOAC_EUNSUPPORTED;
     if (variant_holders(g, v, B) <= 0) return BOAC_ECUDA;
-    const int slots = noalloc_slots(g, v, B);
+    int slots = noalloc_slots(g, v, B);
     if (slots <= 0) return BOAC_EWORKSPACE;  // one candidate's scratch exceeds 64 MiB
+    slots = std::min(slots, split_holders(g, v, B, K));
     void* scratch = noalloc_scratch_ptr();
     if (!scratch) return BOAC_ECUDA;
     // The kernel writes every table entry and sensitivity pixel of a slot
