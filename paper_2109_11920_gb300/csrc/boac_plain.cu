@@ -240,8 +240,9 @@ __global__ void project_table_kernel(int n, int V, float dx, const float* __rest
 // The weights of a pixel's window are the geometry's, so a thread works them
 // out once for C candidates; kViewLanes lanes of a warp take a pixel's views
 // in turn, and every one of them adds up all views' sums in view order (one
-// thread per pixel left the GPU waiting: 4 candidates of 100 x 100 and 75
-// views took 196 us, with 16 lanes and C = 2 62; with 8 lanes 67, C = 4 80).
+// thread per pixel left the GPU waiting where the images are few and small: 4
+// candidates of 100 x 100 and 75 views took 196 us, with 16 lanes and C = 2 62;
+// with 8 lanes 67, C = 4 80).
 template <int C, int kViewLanes>
 __global__ void __launch_bounds__(kPixThreads)
     backproject_gather_kernel(int n, int V, int B, float scale, const float* __restrict__ tab,
@@ -341,15 +342,23 @@ static void gather_launch(int n, int V, int B, float scale, const float* tab, co
 
 void backproject_gather(int n, int V, int B, float scale, const float* tab, const float* y, float* out,
                         int accumulate, cudaStream_t st) {
-    // Two candidates share a thread's weights; a pixel's views go to 16 lanes
-    // while 8 would leave the SMs short of threads (about 1300 each; 6
-    // candidates of 35 x 35 and 109 views, whole call: 0.32 against 0.28 ms;
-    // 5 of 131 x 131: 0.67 against 0.72).
-    const bool wide = (long long)n * n * ((B + 1) / 2) * 8 <= 1300LL * (sm_count() > 0 ? sm_count() : 1);
-    if (B == 1)
-        (wide ? gather_launch<1, 16> : gather_launch<1, 8>)(n, V, B, scale, tab, y, out, accumulate, st);
-    else
-        (wide ? gather_launch<2, 16> : gather_launch<2, 8>)(n, V, B, scale, tab, y, out, accumulate, st);
+    // Two candidates share a thread's weights, and a pixel's views go to as few
+    // lanes as leave the SMs enough threads (about 1600 each): more lanes idle
+    // where the views do not fill their last turn, and each adds up all views'
+    // sums.  (Whole back-projections, us with 1 / 2 / 4 / 8 / 16 lanes: 64 images
+    // of 200 x 200 and 9 views 390 / 445 / 540 / 729 / 978, of 100 x 100 and 75
+    // views 788 / 743 / 742 / 809 / 931; 8 of 150 x 150 and 75 276 / 270 / 235 /
+    // 240 / 270; 4 of 100 x 100 and 75 209 / 131 / 101 / 103 / 100.)
+    const long long items = (long long)n * n * ((B + 1) / 2), want = 1600LL * (sm_count() > 0 ? sm_count() : 1);
+    int lanes = 1;
+    while (lanes < 16 && items * lanes < want) lanes *= 2;
+#define X(L)                                                                                                   \
+    if (lanes == L) {                                                                                          \
+        (B == 1 ? gather_launch<1, L> : gather_launch<2, L>)(n, V, B, scale, tab, y, out, accumulate, st); \
+        return;                                                                                                \
+    }
+    X(1) X(2) X(4) X(8) X(16)
+#undef X
 }
 
 __global__ void ratio_kernel(int count, const float* __restrict__ S, const float* __restrict__ q,
