@@ -96,12 +96,23 @@ __global__ void project_otf_kernel(int n, int V, float dx, const float* __restri
 // where they fit: blockDim.y views of one candidate per CTA, a thread per ray.
 // Same operations and sums.  4 candidates of 100 x 100 and 75 views: a
 // projection from the table took 52 us through L1, here 35.
-__device__ __forceinline__ const float* padded_image(float* smem, int slot, int n, const float* __restrict__ src) {
-    const int P = n + 1, size = P * (n + 2) + 1;
+// A warp's 32 samples are 32 steps along a line across the image, at any angle:
+// at pitch P the cell (row w, column u) lies in bank P w + u, so a line along a
+// short vector of the lattice P w + u = 0 (mod 32) falls on few banks.  Sides that
+// are multiples of 32 would have P = n + 1 = 1 (mod 32) and the vector (1, -1): 20-odd
+// lanes on a bank around 45 and 135 degrees.  ray_pitch takes the next pitch whose
+// shortest vector is at least 5 cells long (us of boac_project, 64 images: 128 x
+// 128 and 75 views 325 -> 248, 96 x 96 and 75 216 -> 142; one image of 128 x 128
+// and 511 views 155 -> 69, 100 x 100, whose pitch was good, 54).
+__device__ __forceinline__ const float* padded_image(float* smem, int slot, int n, int P, const float* __restrict__ src) {
+    const int size = P * (n + 2) + 1;
     float* img = smem + slot * size;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;
     for (int i = tid; i < P; i += nt) img[i] = img[(n + 1) * P + i] = 0.0f;
-    for (int i = tid; i <= n + 1; i += nt) img[i * P] = 0.0f;
+    for (int i = tid; i <= n + 1; i += nt) {
+        img[i * P] = 0.0f;
+        if (P > n + 1) img[i * P + n + 1] = 0.0f;  // else the next row's left padding
+    }
     if (tid == 0) img[size - 1] = 0.0f;
     const int j = threadIdx.x;  // blockDim.x >= n
 #pragma unroll 8
@@ -109,16 +120,17 @@ __device__ __forceinline__ const float* padded_image(float* smem, int slot, int 
         if (j < n) img[(r + 1) * P + j + 1] = __ldg(src + (size_t)r * n + j);
     return img;
 }
-__device__ __forceinline__ float ray_sample_padded(const float* img, int n, int k, int b, float cs, float sn, float c) {
+__device__ __forceinline__ float ray_sample_padded(const float* img, int n, int P, int k, int b, float cs, float sn,
+                                                   float c) {
     float u, w;
     sample_uw(k, b, cs, sn, c, &u, &w);
-    return bilerp_padded(img, n + 1, n, u, w);
+    return bilerp_padded(img, P, n, u, w);
 }
 
 constexpr int kRayViews = 8;  // most views of a CTA
 enum class RayOp { kTable, kProjectTable, kProject };
 template <RayOp OP>
-__global__ void __launch_bounds__(1024) ray_smem_kernel(int n, int V, float dx, const float* __restrict__ mu,
+__global__ void __launch_bounds__(1024) ray_smem_kernel(int n, int P, int V, float dx, const float* __restrict__ mu,
                                                        const float* __restrict__ F, const float* __restrict__ tab,
                                                        float* __restrict__ out) {
     extern __shared__ float smem[];
@@ -127,8 +139,8 @@ __global__ void __launch_bounds__(1024) ray_smem_kernel(int n, int V, float dx, 
     const float* m_img = nullptr;
     const float* f_img = nullptr;
     int slots = 0;
-    if (OP != RayOp::kProjectTable) m_img = padded_image(smem, slots++, n, mu + cand * nn);
-    if (OP != RayOp::kTable) f_img = padded_image(smem, slots++, n, F + cand * nn);
+    if (OP != RayOp::kProjectTable) m_img = padded_image(smem, slots++, n, P, mu + cand * nn);
+    if (OP != RayOp::kTable) f_img = padded_image(smem, slots++, n, P, F + cand * nn);
     __shared__ float csn[kRayViews][2];  // one float64 sine and cosine per view, not per thread
     if (b == 0) view_cos_sin(v, V, &csn[threadIdx.y][0], &csn[threadIdx.y][1]);
     __syncthreads();
@@ -139,7 +151,7 @@ __global__ void __launch_bounds__(1024) ray_smem_kernel(int n, int V, float dx, 
     float suffix = 0.0f, acc = 0.0f;
     if constexpr (OP == RayOp::kTable) {
         walk_ray<8>(
-            n, [&](int k) { return ray_sample_padded(m_img, n, k, b, cs, sn, c); },
+            n, [&](int k) { return ray_sample_padded(m_img, n, P, k, b, cs, sn, c); },
             [&](int k, float m) {
                 out[plane + (size_t)k * n + b] = expf(-dx * (0.5f * m + suffix));
                 suffix += m;
@@ -149,15 +161,15 @@ __global__ void __launch_bounds__(1024) ray_smem_kernel(int n, int V, float dx, 
         walk_ray<8>(
             n,
             [&](int k) {
-                return make_float2(__ldg(tab + plane + (size_t)k * n + b), ray_sample_padded(f_img, n, k, b, cs, sn, c));
+                return make_float2(__ldg(tab + plane + (size_t)k * n + b), ray_sample_padded(f_img, n, P, k, b, cs, sn, c));
             },
             [&](int, float2 s) { acc = fmaf(s.x, s.y, acc); });
     } else {
         walk_ray<4>(
             n,
             [&](int k) {
-                return make_float2(ray_sample_padded(m_img, n, k, b, cs, sn, c),
-                                   ray_sample_padded(f_img, n, k, b, cs, sn, c));
+                return make_float2(ray_sample_padded(m_img, n, P, k, b, cs, sn, c),
+                                   ray_sample_padded(f_img, n, P, k, b, cs, sn, c));
             },
             [&](int, float2 s) {
                 const float a = expf(-dx * (0.5f * s.x + suffix));
@@ -168,6 +180,22 @@ __global__ void __launch_bounds__(1024) ray_smem_kernel(int n, int V, float dx, 
     out[((size_t)cand * V + v) * n + b] = dx * acc;
 }
 
+// The pitch of a padded image of side n (at least n + 1), `images` of which go
+// into shared memory together: see padded_image.  n + 1 where a better one does
+// not fit.
+constexpr size_t kRaySmem = 226 * 1024;
+static size_t ray_smem_bytes(int n, int P, int images) {
+    return sizeof(float) * images * ((size_t)P * (n + 2) + 1);
+}
+static int ray_pitch(int n, int images) {
+    // residues mod 32 with no lattice vector shorter than 5
+    constexpr unsigned kSpread = 1u << 5 | 1u << 6 | 1u << 7 | 1u << 9 | 1u << 12 | 1u << 13 | 1u << 19 | 1u << 20 |
+                                 1u << 23 | 1u << 25 | 1u << 26 | 1u << 27;
+    int P = n + 1;
+    while (!(kSpread >> (P % 32) & 1)) ++P;
+    return ray_smem_bytes(n, P, images) <= kRaySmem ? P : n + 1;
+}
+
 // Launches it where `images` padded images fit an SM, with enough views per CTA
 // to fill it; false: not launched (use the kernels that read global memory).
 template <RayOp OP>
@@ -176,15 +204,16 @@ static bool ray_smem_launch(int n, int V, int B, float dx, const float* mu, cons
     constexpr int kDev = 64;
     static int allowed[kDev];
     const int images = OP == RayOp::kProject ? 2 : 1;
-    const size_t smem = sizeof(float) * images * ((size_t)(n + 1) * (n + 2) + 1);
-    if (smem > 226 * 1024) return false;
+    const int P = ray_pitch(n, images);
+    const size_t smem = ray_smem_bytes(n, P, images);
+    if (smem > kRaySmem) return false;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDev) {
         cudaGetLastError();
         return false;
     }
     if (!allowed[dev]) {
-        if (cudaFuncSetAttribute(ray_smem_kernel<OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) !=
+        if (cudaFuncSetAttribute(ray_smem_kernel<OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRaySmem) !=
             cudaSuccess) {
             cudaGetLastError();
             return false;
@@ -198,7 +227,7 @@ static bool ray_smem_launch(int n, int V, int B, float dx, const float* mu, cons
     if (views > kRayViews) views = kRayViews;
     if (views < 1) views = 1;
     if (views > V) views = V;
-    ray_smem_kernel<OP><<<dim3((V + views - 1) / views, B), dim3(width, views), smem, st>>>(n, V, dx, mu, F, tab, out);
+    ray_smem_kernel<OP><<<dim3((V + views - 1) / views, B), dim3(width, views), smem, st>>>(n, P, V, dx, mu, F, tab, out);
     return true;
 }
 
