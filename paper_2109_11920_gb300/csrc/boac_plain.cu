@@ -23,9 +23,23 @@ namespace cg = cooperative_groups;
 
 namespace boac {
 
+// The ray kernels below read images too large for shared memory through L1, a
+// warp per CTA: where a view's rays run along the rows, a warp's loads touch 32
+// lines each, and the CTAs of that view bound the call, so they have to lie on
+// many SMs (one image of 256 x 256, us of boac_project with 128 / 64 / 32 threads
+// per CTA: 60 views 181 / 119 / 107, 90 views 142 / 113 / 103; 32 images and 60
+// views 999 / 1010 / 805).
+constexpr int kRayGlobalThreads = 32;
+static dim3 ray_global_grid(const boac_geom* g, int B) {
+    return dim3((g->n + kRayGlobalThreads - 1) / kRayGlobalThreads, g->n_views, B);
+}
+
 // Walks a ray from the detector side (k = n - 1) inwards: use(k, load(k)) in
 // order, the loads of DEPTH samples in flight at a time (a sample's four
-// neighbours are an L1 or L2 latency away, and one thread's ray is serial).
+// neighbours are an L1 or L2 latency away, and one thread's ray is serial).  Two
+// where mu is integrated from global memory (one image of 256 x 256, table and
+// back-projection with 1 / 2 / 4 / 8: 9 views 106 / 103 / 126 / 104 us, 60 views
+// 166 / 164 / 188 / 166).
 template <int DEPTH = 4, class Load, class Use>
 __device__ __forceinline__ void walk_ray(int n, Load load, Use use) {
     int k = n - 1;
@@ -58,7 +72,7 @@ __global__ void attenuation_table_kernel(int n, int V, float dx, const float* __
     if (b >= n) return;
     const float c = 0.5f * (float)(n - 1);
     float suffix = 0.0f;
-    walk_ray(
+    walk_ray<2>(
         n, [&](int k) { return ray_sample(m_img, n, k, b, cs, sn, c); },
         [&](int k, float m) {
             t[(size_t)k * n + b] = expf(-dx * (0.5f * m + suffix));
@@ -78,7 +92,7 @@ __global__ void project_otf_kernel(int n, int V, float dx, const float* __restri
     if (b >= n) return;
     const float c = 0.5f * (float)(n - 1);
     float suffix = 0.0f, acc = 0.0f;
-    walk_ray(
+    walk_ray<2>(
         n,
         [&](int k) {
             return make_float2(ray_sample(m_img, n, k, b, cs, sn, c), ray_sample(f_img, n, k, b, cs, sn, c));
@@ -233,16 +247,16 @@ static bool ray_smem_launch(int n, int V, int B, float dx, const float* mu, cons
 
 void attenuation_table(const boac_geom* g, int B, const float* mu, float* tab, cudaStream_t st) {
     if (!ray_smem_launch<RayOp::kTable>(g->n, g->n_views, B, g->pixel_cm, mu, nullptr, nullptr, tab, st))
-        attenuation_table_kernel<<<ray_grid(g, B), kRayThreads, 0, st>>>(g->n, g->n_views, g->pixel_cm, mu, tab);
+        attenuation_table_kernel<<<ray_global_grid(g, B), kRayGlobalThreads, 0, st>>>(g->n, g->n_views, g->pixel_cm, mu, tab);
 }
 void project_rays(const boac_geom* g, int B, const float* mu, const float* F, float* q, cudaStream_t st) {
     if (!ray_smem_launch<RayOp::kProject>(g->n, g->n_views, B, g->pixel_cm, mu, F, nullptr, q, st))
-        project_otf_kernel<<<ray_grid(g, B), kRayThreads, 0, st>>>(g->n, g->n_views, g->pixel_cm, mu, F, q);
+        project_otf_kernel<<<ray_global_grid(g, B), kRayGlobalThreads, 0, st>>>(g->n, g->n_views, g->pixel_cm, mu, F, q);
 }
 void project_table_rays(const boac_geom* g, int B, float dx, const float* tab, const float* F, float* q,
                         cudaStream_t st) {
     if (!ray_smem_launch<RayOp::kProjectTable>(g->n, g->n_views, B, dx, nullptr, F, tab, q, st))
-        project_table_kernel<<<ray_grid(g, B), kRayThreads, 0, st>>>(g->n, g->n_views, dx, tab, F, q);
+        project_table_kernel<<<ray_global_grid(g, B), kRayGlobalThreads, 0, st>>>(g->n, g->n_views, dx, tab, F, q);
 }
 
 // q = A F with a precomputed attenuation table
