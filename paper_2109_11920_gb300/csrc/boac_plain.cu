@@ -386,15 +386,18 @@ static void gather_launch(int n, int V, int B, float scale, const float* tab, co
 void backproject_gather(int n, int V, int B, float scale, const float* tab, const float* y, float* out,
                         int accumulate, cudaStream_t st) {
     // Two candidates share a thread's weights, and a pixel's views go to as few
-    // lanes as leave the SMs enough threads (about 1600 each): more lanes idle
-    // where the views do not fill their last turn, and each adds up all views'
-    // sums.  (Whole back-projections, us with 1 / 2 / 4 / 8 / 16 lanes: 64 images
-    // of 200 x 200 and 9 views 390 / 445 / 540 / 729 / 978, of 100 x 100 and 75
-    // views 788 / 743 / 742 / 809 / 931; 8 of 150 x 150 and 75 276 / 270 / 235 /
-    // 240 / 270; 4 of 100 x 100 and 75 209 / 131 / 101 / 103 / 100.)
-    const long long items = (long long)n * n * ((B + 1) / 2), want = 1600LL * (sm_count() > 0 ? sm_count() : 1);
+    // lanes as leave the SMs enough threads: more lanes idle where the views do
+    // not fill their last turn, and each adds up all views' sums.  That is about
+    // 1600 threads each, or 3400 from 32 views on, where the turns are full, with
+    // 16 lanes only for what 8 leave below 1600.  (Whole back-projections, us with
+    // 1 / 2 / 4 / 8 / 16 lanes: 64 images of 200 x 200 and 9 views 390 / 445 / 540 /
+    // 729 / 978, 64 of 100 x 100 and 120 views 1229 / 1149 / 1138 / 1185 / 1394; 8 of
+    // 200 x 200 and 240 1527 / 1306 / 1211 / 1217 / 1338, 8 of 100 x 100 and 75 218 /
+    // 155 / 151 / 140 / 144; 4 of 100 x 100 and 75 209 / 131 / 101 / 103 / 100.)
+    const long long items = (long long)n * n * ((B + 1) / 2), sms = sm_count() > 0 ? sm_count() : 1;
     int lanes = 1;
-    while (lanes < 16 && items * lanes < want) lanes *= 2;
+    while (lanes < 8 && items * lanes < (V < 32 ? 1600 : 3400) * sms) lanes *= 2;
+    if (lanes == 8 && items * 8 < 1600 * sms) lanes = 16;
 #define X(L)                                                                                                   \
     if (lanes == L) {                                                                                          \
         (B == 1 ? gather_launch<1, L> : gather_launch<2, L>)(n, V, B, scale, tab, y, out, accumulate, st); \

@@ -1,6 +1,6 @@
 """The per-pixel back-projection with 1 to 16 lanes per pixel: batches that take
-each (images and candidates enough for 243 200 threads on 152 SMs), odd sides,
-odd batches and fewer views than lanes.  A pixel's views are added up in order
+each (images and candidates enough for 243 200 threads on 152 SMs, 516 800 from
+32 views on), odd sides, odd batches and fewer views than lanes.  A pixel's views are added up in order
 whichever lanes take them, so a batch's images are those of one-candidate
 calls, which take other lanes, bit for bit (the operators' tests compare those
 with the oracle).  And one view more than a turn of 8 lanes costs a large batch
@@ -15,7 +15,9 @@ pytestmark = pytest.mark.gpu
 
 
 # lanes of the batch:                          1             1            2            4           8           16
-@pytest.mark.parametrize("n,V,B", [(181, 3, 15), (100, 17, 49), (181, 9, 7), (101, 5, 13), (65, 21, 15), (33, 7, 3)])
+@pytest.mark.parametrize("n,V,B", [(181, 3, 15), (100, 17, 49), (181, 9, 7), (101, 5, 13), (65, 21, 15), (33, 7, 3),
+                                   (201, 33, 29), (181, 33, 15), (181, 32, 7), (65, 33, 31), (65, 45, 9)])
+# and from 32 views on:               1              2             4            8            16
 def test_lanes_give_the_same_bits(cuda, n, V, B):
     g = Geom.make(n, 25.6 / n, V)
     gen = torch.Generator(device=cuda).manual_seed(n + V)
