@@ -7,8 +7,8 @@
 // once per view through L1 with 128 dependent steps, and the table-based
 // back-projector writes and reads every attenuation factor (8 MB per candidate
 // at 128 x 128 and 120 views); other sizes still use them (boac_plain.cu).
-// Measured, 64 candidates at 128 x 128 and 120 views: projection 128 us
-// (880), back-projection 171 us (780).
+// Measured, 64 candidates at 128 x 128 and 120 views: projection 126 us
+// (880), back-projection 165 us (780).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -53,9 +53,13 @@ __device__ __forceinline__ void segment_sums(const float* part, int lb, int seg,
     *after = a;
 }
 
-// 2^x, results below 2^-126 kept (ex2 flushes them to 0, up to 27 % of a pixel
-// behind 60 cm at 8 / cm; 2 % of the operators' time).
+// 2^x.  TINY: results below 2^-126 kept (ex2 flushes them to 0: up to 27 % of a
+// pixel behind 60 cm at 8 / cm).  Only the CTAs whose mu can lead there do (see
+// load_scaled); on all, the operators on 64 images take 128 + 171 us instead of
+// 126 + 165.
+template <bool TINY>
 __device__ __forceinline__ float factor(float x) {
+    if constexpr (!TINY) return ex2(x);
     float y;
     asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
@@ -64,16 +68,16 @@ __device__ __forceinline__ float factor(float x) {
 // A thread's run of SEG samples m of a ray, scaled for base 2 (load_scaled):
 // the factors towards the ray's end (e[2 s]: the half-cell sum of the samples
 // behind it) and towards its start (e[2 s + 1]).
-template <int SEG>
+template <bool TINY, int SEG>
 __device__ __forceinline__ void run_factors(const float (&m)[SEG], float before, float after, float (&e)[2 * SEG]) {
 #pragma unroll
     for (int s = 0; s < SEG; ++s) {
-        e[2 * s + 1] = factor(fmaf(0.5f, m[s], before));
+        e[2 * s + 1] = factor<TINY>(fmaf(0.5f, m[s], before));
         before += m[s];
     }
 #pragma unroll
     for (int s = SEG - 1; s >= 0; --s) {
-        e[2 * s] = factor(fmaf(0.5f, m[s], after));
+        e[2 * s] = factor<TINY>(fmaf(0.5f, m[s], after));
         after += m[s];
     }
 }
@@ -90,44 +94,37 @@ __device__ __forceinline__ void load_image(float* img, const float* __restrict__
 // every attenuation factor: back-projections at 128 x 128, 120 views and 2 / cm
 // were 9.5e-7 off (root mean square of the pixels' relative errors against 64
 // bits), now 9.0e-7; with expf of the sum 9.0e-7 and 160 + 196 us instead of
-// 128 + 171 for both operators on 64 images.
+// 126 + 165 for the operators on 64 images.  (The factor comes from the host:
+// its float64 product by each of 1024 threads takes 1 us.)
+//
+// Returns whether a factor below 2^-126 is possible: an exponent is at most the
+// sum of a ray's samples, N times the largest |mu| (to rounding, 125 for 126).
+// Called by all threads; ends with a barrier.
 template <int N, int NT, int P>
-__device__ __forceinline__ void load_scaled(float* img, const float* __restrict__ src, float dx) {
-    const double s = -1.44269504088896340736 * (double)dx;
-    const float hi = (float)s, lo = (float)(s - (double)hi);
+__device__ __forceinline__ bool load_scaled(float* img, const float* __restrict__ src, float2 scale) {
+    bool dense = false;
 #pragma unroll 4
     for (int i = threadIdx.x; i < N * N; i += NT) {
-        const float v = __ldg(src + i);
-        img[(i / N + 1) * P + (i % N) + 1] = fmaf(v, hi, v * lo);
+        const float v = __ldg(src + i), x = fmaf(v, scale.x, v * scale.y);
+        img[(i / N + 1) * P + (i % N) + 1] = x;
+        dense |= !(fabsf(x) < 125.0f / N);  // (or not a number)
     }
+    return __syncthreads_or(dense);
 }
 
-// q of grids [blockIdx.x share) of candidate blockIdx.y.  Bounded by the two
-// gathers of every sample (shared memory) and the barriers between the column
-// and row passes, as the fused MLEM kernel's forward half.
-template <int N, bool QUAD>
-__global__ void __launch_bounds__(8 * N, 1)
-    project_grids_kernel(int V, float dx, const float* __restrict__ mu, const float* __restrict__ F,
-                         float* __restrict__ q) {
+// q of one candidate's grids [g0, g1), their directions in csn, its images in
+// shared memory.
+template <int N, bool QUAD, bool TINY>
+__device__ __forceinline__ void project_grids(int V, float dx, int g0, int g1, const float* csn, float* smem,
+                                              float* __restrict__ q) {
     using O = OpShape<N>;
     constexpr int NT = O::NT, P = O::P, WP = O::WP, IMG = O::IMG, NSEG = O::NSEG, SEG = O::SEG;
-    extern __shared__ __align__(16) float smem[];
-    float* img0 = smem;             // F
-    float* img1 = img0 + IMG;       // mu, scaled
-    float* W = img1 + IMG;          // [N][WP] samples of mu, then of F
-    float* red = W + N * WP;        // [4][NSEG][N]
+    const float* img0 = smem;        // F
+    const float* img1 = img0 + IMG;  // mu, scaled
+    float* W = smem + 2 * IMG;       // [N][WP] samples of mu, then of F
+    float* red = W + N * WP;         // [4][NSEG][N]
     const int tid = threadIdx.x, lb = tid % N, seg = tid / N, k0 = seg * SEG;
-    const int cand = blockIdx.y, ngrid = QUAD ? V / 4 : V / 2;
-    const int g0 = (int)((long long)blockIdx.x * ngrid / gridDim.x);
-    const int g1 = (int)((long long)(blockIdx.x + 1) * ngrid / gridDim.x);
     const float c = 0.5f * (float)(N - 1);
-    __shared__ float csn[kMaxViews];  // the share's grids (at most half the views)
-    for (int gi = g0 + tid; gi < g1; gi += NT) view_cos_sin(gi, V, &csn[2 * (gi - g0)], &csn[2 * (gi - g0) + 1]);
-    for (int i = tid; i < 2 * IMG; i += NT) smem[i] = 0.0f;
-    __syncthreads();
-    load_image<N, NT, P>(img0, F + (size_t)cand * N * N);
-    load_scaled<N, NT, P>(img1, mu + (size_t)cand * N * N, dx);
-    __syncthreads();
     for (int gi = g0; gi < g1; ++gi) {
         const float cs = csn[2 * (gi - g0)], sn = csn[2 * (gi - g0) + 1];
         float f[SEG], e[2 * SEG];
@@ -149,7 +146,7 @@ __global__ void __launch_bounds__(8 * N, 1)
             __syncthreads();
             float before, after;
             segment_sums<N, NSEG>(red, lb, seg, &before, &after);
-            run_factors<SEG>(m, before, after, e);
+            run_factors<TINY, SEG>(m, before, after, e);
         }
         float a1 = 0.0f, a2 = 0.0f;
 #pragma unroll
@@ -172,7 +169,7 @@ __global__ void __launch_bounds__(8 * N, 1)
             __syncthreads();
             float before, after;
             segment_sums<N, NSEG>(red + NSEG * N, lb, seg, &before, &after);
-            run_factors<SEG>(m, before, after, e);
+            run_factors<TINY, SEG>(m, before, after, e);
 #pragma unroll
             for (int s = 0; s < SEG; ++s) W[(k0 + s) * WP + lb] = f[s];
             __syncthreads();
@@ -201,46 +198,55 @@ __global__ void __launch_bounds__(8 * N, 1)
             float sum = 0.0f;
 #pragma unroll
             for (int s = 0; s < NSEG; ++s) sum += red[(vi * NSEG + s) * N + j];
-            q[((size_t)cand * V + grid_view<QUAD>(gi, vi, V)) * N + grid_bin<N>(vi, j)] = dx * sum;
+            q[(size_t)grid_view<QUAD>(gi, vi, V) * N + grid_bin<N>(vi, j)] = dx * sum;
         }
         __syncthreads();
     }
 }
 
-// z of grids [blockIdx.x share) of candidate blockIdx.y into its partial
-// image.  SCHED: the scatter runs in the order of a kept schedule; elsewhere
-// in lattice order, with the same sums (one image at 128 x 128 and 120 views: a
-// schedule of the call's own takes about 190 us to build, all else 33 us;
-// 8 images with 230 views in lattice order, both operators: 297 us, with the
-// per-ray and per-grid table kernels 630).
-template <int N, bool QUAD, bool SCHED>
+// q of grids [blockIdx.x share) of candidate blockIdx.y.  Bounded by the two
+// gathers of every sample (shared memory) and the barriers between the column
+// and row passes, as the fused MLEM kernel's forward half.
+template <int N, bool QUAD>
 __global__ void __launch_bounds__(8 * N, 1)
-    backproject_grids_kernel(int V, float dx, const float* __restrict__ mu, const float* __restrict__ y,
-                             const unsigned short* __restrict__ sched, float* __restrict__ partial) {
+    project_grids_kernel(int V, float dx, float2 scale, const float* __restrict__ mu, const float* __restrict__ F,
+                         float* __restrict__ q) {
     using O = OpShape<N>;
-    constexpr int NT = O::NT, P = O::P, WP = O::WP, IMG = O::IMG, NSEG = O::NSEG, SEG = O::SEG;
+    constexpr int NT = O::NT, P = O::P, IMG = O::IMG;
     extern __shared__ __align__(16) float smem[];
-    float* img0 = smem;             // mu, scaled
-    float* img1 = img0 + IMG;       // accumulator
-    float* W = img1 + IMG;          // [N][WP] samples of mu, then weights
-    float* red = W + N * WP;        // [2][NSEG][N]
-    float* yy = red + 4 * NSEG * N;  // [4][N] dx y by grid coordinate
-    const int tid = threadIdx.x, lb = tid % N, seg = tid / N, k0 = seg * SEG;
-    const int cand = blockIdx.y, ngrid = QUAD ? V / 4 : V / 2;
+    const int tid = threadIdx.x, cand = blockIdx.y, ngrid = QUAD ? V / 4 : V / 2;
     const int g0 = (int)((long long)blockIdx.x * ngrid / gridDim.x);
     const int g1 = (int)((long long)(blockIdx.x + 1) * ngrid / gridDim.x);
-    const float c = 0.5f * (float)(N - 1);
     __shared__ float csn[kMaxViews];  // the share's grids (at most half the views)
     for (int gi = g0 + tid; gi < g1; gi += NT) view_cos_sin(gi, V, &csn[2 * (gi - g0)], &csn[2 * (gi - g0) + 1]);
     for (int i = tid; i < 2 * IMG; i += NT) smem[i] = 0.0f;
     __syncthreads();
-    load_scaled<N, NT, P>(img0, mu + (size_t)cand * N * N, dx);
-    __syncthreads();
+    load_image<N, NT, P>(smem, F + (size_t)cand * N * N);
+    const bool dense = load_scaled<N, NT, P>(smem + IMG, mu + (size_t)cand * N * N, scale);
+    float* qc = q + (size_t)cand * V * N;
+    if (dense) project_grids<N, QUAD, true>(V, dx, g0, g1, csn, smem, qc);
+    else project_grids<N, QUAD, false>(V, dx, g0, g1, csn, smem, qc);
+}
+
+// z of one candidate's grids [g0, g1) into the accumulator img1.
+template <int N, bool QUAD, bool SCHED, bool TINY>
+__device__ __forceinline__ void backproject_grids(int V, float dx, int g0, int g1, const float* csn, float* smem,
+                                                  const float* __restrict__ y,
+                                                  const unsigned short* __restrict__ sched) {
+    using O = OpShape<N>;
+    constexpr int NT = O::NT, P = O::P, WP = O::WP, IMG = O::IMG, NSEG = O::NSEG, SEG = O::SEG;
+    const float* img0 = smem;       // mu, scaled
+    float* img1 = smem + IMG;       // accumulator
+    float* W = img1 + IMG;          // [N][WP] samples of mu, then weights
+    float* red = W + N * WP;        // [2][NSEG][N]
+    float* yy = red + 4 * NSEG * N;  // [4][N] dx y by grid coordinate
+    const int tid = threadIdx.x, lb = tid % N, seg = tid / N, k0 = seg * SEG;
+    const float c = 0.5f * (float)(N - 1);
     for (int gi = g0; gi < g1; ++gi) {
         const float cs = csn[2 * (gi - g0)], sn = csn[2 * (gi - g0) + 1];
         for (int t = tid; t < (QUAD ? 4 : 2) * N; t += NT) {
             const int vi = t / N, j = t % N;
-            yy[t] = dx * (y ? __ldg(y + ((size_t)cand * V + grid_view<QUAD>(gi, vi, V)) * N + grid_bin<N>(vi, j)) : 1.0f);
+            yy[t] = dx * (y ? __ldg(y + (size_t)grid_view<QUAD>(gi, vi, V) * N + grid_bin<N>(vi, j)) : 1.0f);
         }
         float e[2 * SEG], gc[SEG];
         {
@@ -256,7 +262,7 @@ __global__ void __launch_bounds__(8 * N, 1)
             __syncthreads();
             float before, after;
             segment_sums<N, NSEG>(red, lb, seg, &before, &after);
-            run_factors<SEG>(m, before, after, e);
+            run_factors<TINY, SEG>(m, before, after, e);
         }
         {
             const float y1 = yy[lb], y2 = yy[N + lb];
@@ -275,7 +281,7 @@ __global__ void __launch_bounds__(8 * N, 1)
             __syncthreads();
             float before, after;
             segment_sums<N, NSEG>(red + NSEG * N, lb, seg, &before, &after);
-            run_factors<SEG>(m, before, after, e);
+            run_factors<TINY, SEG>(m, before, after, e);
         }
 #pragma unroll
         for (int s = 0; s < SEG; ++s) W[(k0 + s) * WP + lb] = gc[s];
@@ -300,8 +306,40 @@ __global__ void __launch_bounds__(8 * N, 1)
         if constexpr (SCHED) scatter_scheduled<N, NT, P, WP>(W, img1, cs, sn, c, gs, sched0);
         else scatter_classes<N, NT, P, WP>(W, img1, cs, sn, c);
     }
+}
+
+// z of grids [blockIdx.x share) of candidate blockIdx.y into its partial
+// image.  SCHED: the scatter runs in the order of a kept schedule; elsewhere
+// in lattice order, with the same sums (one image at 128 x 128 and 120 views: a
+// schedule of the call's own takes about 190 us to build, all else 33 us;
+// 8 images with 230 views in lattice order, both operators: 297 us, with the
+// per-ray and per-grid table kernels 630).
+template <int N, bool QUAD, bool SCHED>
+__global__ void __launch_bounds__(8 * N, 1)
+    backproject_grids_kernel(int V, float dx, float2 scale, const float* __restrict__ mu, const float* __restrict__ y,
+                             const unsigned short* __restrict__ sched, float* __restrict__ partial) {
+    using O = OpShape<N>;
+    constexpr int NT = O::NT, P = O::P, IMG = O::IMG;
+    extern __shared__ __align__(16) float smem[];
+    const int tid = threadIdx.x, cand = blockIdx.y, ngrid = QUAD ? V / 4 : V / 2;
+    const int g0 = (int)((long long)blockIdx.x * ngrid / gridDim.x);
+    const int g1 = (int)((long long)(blockIdx.x + 1) * ngrid / gridDim.x);
+    __shared__ float csn[kMaxViews];  // the share's grids (at most half the views)
+    for (int gi = g0 + tid; gi < g1; gi += NT) view_cos_sin(gi, V, &csn[2 * (gi - g0)], &csn[2 * (gi - g0) + 1]);
+    for (int i = tid; i < 2 * IMG; i += NT) smem[i] = 0.0f;
+    __syncthreads();
+    const bool dense = load_scaled<N, NT, P>(smem, mu + (size_t)cand * N * N, scale);
+    const float* yc = y ? y + (size_t)cand * V * N : nullptr;
+    if (dense) backproject_grids<N, QUAD, SCHED, true>(V, dx, g0, g1, csn, smem, yc, sched);
+    else backproject_grids<N, QUAD, SCHED, false>(V, dx, g0, g1, csn, smem, yc, sched);
     float* out = partial + ((size_t)cand * gridDim.x + blockIdx.x) * N * N;
-    for (int i = tid; i < N * N; i += NT) out[i] = img1[(i / N + 1) * P + (i % N) + 1];
+    for (int i = tid; i < N * N; i += NT) out[i] = smem[IMG + (i / N + 1) * P + (i % N) + 1];
+}
+
+// -dx log2(e) in two floats (load_scaled).
+float2 exponent_scale(float dx) {
+    const double s = -1.44269504088896340736 * (double)dx;
+    return make_float2((float)s, (float)(s - (double)(float)s));
 }
 
 // CTAs per candidate for B candidates of ngrid grids: the least rounds over
@@ -340,7 +378,8 @@ int project_t(int V, float dx, const float* mu, const float* F, int B, float* q,
     const int s = allow_smem(project_grids_kernel<N, QUAD>, OpShape<N>::SMEM, done);
     if (s != BOAC_OK) return s;
     project_grids_kernel<N, QUAD>
-        <<<dim3(grid_shares(B, QUAD ? V / 4 : V / 2), B), 8 * N, OpShape<N>::SMEM, st>>>(V, dx, mu, F, q);
+        <<<dim3(grid_shares(B, QUAD ? V / 4 : V / 2), B), 8 * N, OpShape<N>::SMEM, st>>>(V, dx, exponent_scale(dx), mu,
+                                                                                         F, q);
     return launch_status();
 }
 
@@ -355,7 +394,7 @@ int backproject_t(int V, float dx, const float* mu, const float* y, int B, float
     auto kernel = sched ? backproject_grids_kernel<N, QUAD, true> : backproject_grids_kernel<N, QUAD, false>;
     s = allow_smem(kernel, OpShape<N>::SMEM, done[sched != nullptr]);
     if (s != BOAC_OK) return s;
-    kernel<<<dim3(shares, B), 8 * N, OpShape<N>::SMEM, st>>>(V, dx, mu, y, sched, partial);
+    kernel<<<dim3(shares, B), 8 * N, OpShape<N>::SMEM, st>>>(V, dx, exponent_scale(dx), mu, y, sched, partial);
     return sum_partial_images(B, shares, N * N, partial, out, st);
 }
 
