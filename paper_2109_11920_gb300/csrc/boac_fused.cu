@@ -141,11 +141,13 @@ static const FusedVariant* get_variant(const boac_geom* g, int config);
 // (images up to 128 x 128, V % 4 == 0): the cluster size G with the least
 // modelled time, rounds(G) (ceil(grids / G) + 1.6) grid passes per
 // iteration, where rounds(G) = ceil(B / clusters of G resident at once) and
-// 1.6 grid passes stand for the cluster's per-iteration exchange (fitted on
-// GB300 at 128 x 128 and 120 views: 24 us against 15 us per grid pass); the
+// 1.6 grid passes stand for the cluster's per-iteration exchange; the
 // smaller G on a tie; and only if that beats one CTA per candidate, whose
 // even split of the batch's iterations costs grids B / min(B, SMs) passes
-// per iteration.  Returns the configuration id, or -1.
+// per iteration.  Returns the configuration id, or -1.  (1.6 was fitted to
+// earlier kernels and is high: an iteration at 128 x 128 and 120 views takes
+// 295 us on one CTA, 151 / 81 / 44 / 28 us on G = 2 / 4 / 8 / 16, that is 9.8 us
+// per grid pass and 0.2 to 0.8 passes of exchange.)
 static int split_config(const boac_geom* g, int B) {
     if (g->n > 128 || g->n_views % 4 != 0 || B < 1) return -1;
     const int sms = sm_count();
@@ -171,9 +173,7 @@ static int split_config(const boac_geom* g, int B) {
 
 // Default configuration for B candidates.  Batches too small to fill the
 // GPU one candidate per CTA (images up to 128 x 128, V % 4 == 0) take the
-// fused kernel's cluster mode (split_config; measured on GB300 at 128 x 128
-// and K = 20: 1.7x to 2.3x the unfused batched kernels at 1 to 64
-// candidates, 1.2x the one-CTA kernel at 96).  256 x 256 images with
+// fused kernel's cluster mode (split_config).  256 x 256 images with
 // V % 4 == 0 take the band kernel with the cluster size that keeps the most
 // SMs busy (clusters are placed within one GPC, so the resident count
 // depends on the size); the smaller cluster on a tie.  Otherwise the one-CTA
@@ -182,9 +182,9 @@ static int default_config(const boac_geom* g, int B) {
     const int sc = split_config(g, B);
     if (sc >= 0) return sc;
     if (g->n == 64 && B >= 1 && B <= 2 * sm_count()) {
-        // at most two candidates per SM: CTAs of 8n threads (measured on GB300
-        // at 60 views: 1.88 vs 2.16 ms for B = 1 ... 128; from B = 456 on,
-        // three 4n-thread CTAs per SM are faster)
+        // at most two candidates per SM: CTAs of 8n threads (60 views, us per grid
+        // of a CTA alone on its SM: 4.1, of 4n threads 5.3); beyond, three of 4n
+        // threads per SM (456 candidates x 20 iterations 3.32 ms)
         return 2 * 2 + (g->n_views % 4 == 0 ? 0 : 1);
     }
     if (g->n == 256 && g->n_views % 4 == 0) {
@@ -205,11 +205,13 @@ static int default_config(const boac_geom* g, int B) {
 // Batches small enough that the unfused batched kernels (boac_unfused.cu:
 // many CTAs per candidate) finish before the fused kernel's one CTA or one
 // cluster per candidate does, for the geometries without the cluster mode
-// (view counts not divisible by 4, 256 x 256 images).  Measured on GB300
-// (152 SMs) with K = 20 at 60 / 90 / 120 / 180 views: up to 32 candidates at
-// 64 x 64 and 96 x 96 (1.9x / 4.7x at B = 1), 16 at 128 x 128 (2.4x at
-// B = 1), 2 at 256 x 256 (1.3x at B = 1); both paths scale with the view
-// count, so the bound is per image size, scaled with the SM count.
+// (view counts not divisible by 4, 256 x 256 images): up to 32 candidates at
+// 64 x 64 and 96 x 96, 16 at 128 x 128, 2 at 256 x 256.  Both paths scale with
+// the view count, so the bound is per image size, scaled with the SM count.
+// (The bounds were fitted to earlier kernels and are low: ms of 20 iterations,
+// unfused against fused, 64 x 64 and 90 views 32 candidates 1.42 / 3.84, 64
+// 2.62 / 3.86; 96 x 96 32 2.55 / 5.86; 128 x 128 16 2.67 / 8.87; 256 x 256 and 90
+// views 4 9.5 / 190, 180 views 2 10.0 / 19.3, 4 17.8 / 21.2.)
 static bool use_unfused(const boac_geom* g, int B) {
     if (split_config(g, B) >= 0) return false;
     int cap;
@@ -451,16 +453,16 @@ struct RaggedPlan {
 // of one-CTA candidates needs at least the SMs that finish its work in the
 // time T of the longest chain: T starts at the larger of the longest
 // candidate's time and the even share of all work, and grows until the
-// classes fit the GPU together.  Time per sample grid, measured: 11.1 us at
-// 128 x 128 and 5.3 us at 64 x 64, that is 0.47 ns per sample and as much as
-// 7200 samples for its barriers; two views per grid 0.85 times that (6.5 us
-// at 96 x 96); a second and third CTA on an SM count as 0.45 of one each.  (They
+// classes fit the GPU together.  Time per sample grid, modelled as that of its
+// samples and of 7200 more for its barriers (0.36 to 0.42 ns each: 9.9 us at 128 x
+// 128, 6.8 at 96 x 96, 4.1 at 64 x 64); two views per grid 0.85 times that (8.9,
+// 6.1, 4.5 us); a second and third CTA on an SM count as 0.45 of one each.  (They
 // take 0.6 and 0.75: 64 x 64, 60 views, 20 iterations of 152, 304 and 456
 // candidates 1.41, 2.28 and 3.32 ms.  With 0.65, batches take longer: 600 beside
 // 152 of 128 x 128 13.6 against 12.6 ms, 128 beside 128 8.8 against 7.3.)
 //
 // The one-CTA kernel at 256 x 256 keeps its images in global memory and slows
-// down with the CTAs that share L2: 200, 339 and 521 us per grid of two views
+// down with the CTAs that share L2: 200, 320 and 525 us per grid of two views
 // with 8, 64 and 152 of them, 6.6 times the time of a kernel with its images on
 // chip and 0.085 more per CTA.  Up to kSharedGlobalCtas such CTAs run beside
 // the other classes (32 candidates of 90 views and 16 of 180: 118 ms, one class

@@ -118,7 +118,8 @@ __global__ void project_otf_kernel(int n, int V, float dx, const float* __restri
 // shortest vector is at least 5 cells long (us of boac_project, 64 images: 128 x
 // 128 and 75 views 325 -> 248, 96 x 96 and 75 216 -> 142; one image of 128 x 128
 // and 511 views 155 -> 69, 100 x 100, whose pitch was good, 54).
-__device__ __forceinline__ const float* padded_image(float* smem, int slot, int n, int P, const float* __restrict__ src) {
+__device__ __forceinline__ const float* padded_image(float* smem, int slot, int n, int P,
+                                                     const float* __restrict__ src) {
     const int size = P * (n + 2) + 1;
     float* img = smem + slot * size;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;
@@ -175,7 +176,8 @@ __global__ void __launch_bounds__(1024) ray_smem_kernel(int n, int P, int V, flo
         walk_ray<8>(
             n,
             [&](int k) {
-                return make_float2(__ldg(tab + plane + (size_t)k * n + b), ray_sample_padded(f_img, n, P, k, b, cs, sn, c));
+                return make_float2(__ldg(tab + plane + (size_t)k * n + b),
+                                   ray_sample_padded(f_img, n, P, k, b, cs, sn, c));
             },
             [&](int, float2 s) { acc = fmaf(s.x, s.y, acc); });
     } else {
@@ -241,17 +243,20 @@ static bool ray_smem_launch(int n, int V, int B, float dx, const float* mu, cons
     if (views > kRayViews) views = kRayViews;
     if (views < 1) views = 1;
     if (views > V) views = V;
-    ray_smem_kernel<OP><<<dim3((V + views - 1) / views, B), dim3(width, views), smem, st>>>(n, P, V, dx, mu, F, tab, out);
+    ray_smem_kernel<OP>
+        <<<dim3((V + views - 1) / views, B), dim3(width, views), smem, st>>>(n, P, V, dx, mu, F, tab, out);
     return true;
 }
 
 void attenuation_table(const boac_geom* g, int B, const float* mu, float* tab, cudaStream_t st) {
     if (!ray_smem_launch<RayOp::kTable>(g->n, g->n_views, B, g->pixel_cm, mu, nullptr, nullptr, tab, st))
-        attenuation_table_kernel<<<ray_global_grid(g, B), kRayGlobalThreads, 0, st>>>(g->n, g->n_views, g->pixel_cm, mu, tab);
+        attenuation_table_kernel<<<ray_global_grid(g, B), kRayGlobalThreads, 0, st>>>(g->n, g->n_views, g->pixel_cm, mu,
+                                                                                      tab);
 }
 void project_rays(const boac_geom* g, int B, const float* mu, const float* F, float* q, cudaStream_t st) {
     if (!ray_smem_launch<RayOp::kProject>(g->n, g->n_views, B, g->pixel_cm, mu, F, nullptr, q, st))
-        project_otf_kernel<<<ray_global_grid(g, B), kRayGlobalThreads, 0, st>>>(g->n, g->n_views, g->pixel_cm, mu, F, q);
+        project_otf_kernel<<<ray_global_grid(g, B), kRayGlobalThreads, 0, st>>>(g->n, g->n_views, g->pixel_cm, mu, F,
+                                                                                q);
 }
 void project_table_rays(const boac_geom* g, int B, float dx, const float* tab, const float* F, float* q,
                         cudaStream_t st) {
