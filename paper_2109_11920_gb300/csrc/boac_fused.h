@@ -100,7 +100,8 @@ __device__ __forceinline__ void class_end(const FusedArgs& a) {
 // however long the candidate is.  (The first part's CTA starts no later: CTAs
 // are dispatched in index order.)
 __device__ __forceinline__ long long wait_limit(const FusedArgs& a, long long u0, long long setup) {
-    return a.wait_cycles + 4 * u0 * setup;
+    const long long first = 4 * u0 * setup, room = 0x7fffffffffffffffLL - first;
+    return first + (a.wait_cycles < room ? a.wait_cycles : room);  // wait_cycles may be any positive number
 }
 // Element i of every rank's copy of a shared-memory array, summed in rank
 // order; and the same value stored into every rank's copy.  All the loads are

@@ -43,3 +43,17 @@ def test_long_first_part_is_no_timeout(cuda, parts, config):
         finally:
             boac.boac_set_wait_cycles(old)
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+def test_largest_limit(cuda):
+    """The largest limit that can be set never runs out."""
+    g, B, K = Geom.make(64, 0.4, 60), 229, 7
+    mu = torch.full((64, 64), 0.1, device=cuda)
+    S = torch.ones(60, 64, device=cuda)
+    b = boac.RaggedBatch([g], [0] * B, [K + i % 3 for i in range(B)], [mu] * B, [S] * B, device=cuda)
+    old = boac.boac_set_wait_cycles(2**63 - 1)
+    try:
+        L = boac.boac_mlem_ragged(b, config=[2])  # raises where a wait gave up
+    finally:
+        boac.boac_set_wait_cycles(old)
+    assert bool(torch.isfinite(L).all())
