@@ -105,7 +105,8 @@ __device__ __forceinline__ bool load_scaled(float* img, const float* __restrict_
     bool dense = false;
 #pragma unroll 4
     for (int i = threadIdx.x; i < N * N; i += NT) {
-        const float v = __ldg(src + i), x = fmaf(v, scale.x, v * scale.y);
+        const float v = __ldg(src + i);
+        const float x = fabsf(v) < INFINITY ? fmaf(v, scale.x, v * scale.y) : v * scale.x;  // (inf - inf is not inf)
         img[(i / N + 1) * P + (i % N) + 1] = x;
         dense |= !(fabsf(x) < 125.0f / N);  // (or not a number)
     }
